@@ -137,29 +137,20 @@ bool any_config_valid(int N, int NT, iqa_dtype dtype, const TileConfig &c,
     return false;
 }
 
-// CTAs of the tile kernel in shape c that one SM holds at once (0 if the
-// runtime cannot tell), cached per context.
-static int tiles_occupancy(iqa_ctx *ctx, iqa_dtype dtype, const TileConfig &c, int maps)
+// CTAs per SM that the one-wave rule below counts with.  A launch shape fixes
+// the order of a tile's sums, so these numbers are part of a map's bits: they
+// are those of the kernel whose shapes were swept for the rule (96 to 120
+// registers a thread with eight FP32 vectors in flight, 46 to 72 otherwise) and
+// stay as they are whatever the kernel's registers or shared memory become.
+static int shape_residency(iqa_dtype dtype, const TileConfig &c)
 {
-    const auto key = std::make_tuple((int)dtype, c.vec * 1000 + c.ilp, c.threads, maps);
-    {
-        std::lock_guard<std::mutex> g(ctx->cfg_mu);
-        auto it = ctx->occupancy.find(key);
-        if (it != ctx->occupancy.end()) return it->second;
+    if (dtype == IQA_F32) {
+        const int deep[3] = {5, 2, 1}, shallow[3] = {10, 5, 2};
+        return (c.ilp == 8 ? deep : shallow)[c.threads / 256];
     }
-    TileArgs none;
-    std::memset(&none, 0, sizeof none);
-    int occ = 0;
-    cudaError_t e = dtype == IQA_F32   ? launch_tiles_f32(none, c, maps, 0, nullptr, &occ)
-                    : dtype == IQA_F16 ? launch_tiles_f16(none, c, maps, 0, nullptr, &occ)
-                                       : launch_tiles_bf16(none, c, maps, 0, nullptr, &occ);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        occ = 0;
-    }
-    std::lock_guard<std::mutex> g(ctx->cfg_mu);
-    ctx->occupancy[key] = occ;
-    return occ;
+    if (c.threads == 128) return c.ilp == 8 ? 10 : 9;
+    if (c.threads == 256) return c.ilp == 2 ? 5 : 4;
+    return dtype == IQA_BF16 && c.ilp == 4 ? 1 : 2;
 }
 
 // Launch shape when nothing was tuned (measured on GB300: 128-thread CTAs
@@ -228,12 +219,10 @@ TileConfig default_config(int N, int NT, iqa_dtype dtype, bool aligned,
 // most two waves of resident CTAs (the last wave then runs a fraction of the
 // GPU and its ramp and tail are paid twice), units twice as wide that fit one
 // wave are used instead (N=2048, N_T=64: 512 CTAs of two tiles, 12.96 against
-// 14.3 us per isolated launch).  Residency is that of the kernel forming both
-// maps (the most registers), whichever maps are requested, so that a map comes
-// out of the same launch shape, and so bit for bit the same, in every call.
+// 14.3 us per isolated launch).  A map comes out of the same launch shape, and
+// so bit for bit the same, in every call, whichever maps are requested.
 static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, TileConfig c)
 {
-    const int maps = MAPS_AB;
     if (c.variant != 0 || c.S != 1 || c.vec == 1) return c;
     const int T = N / NT;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
@@ -243,8 +232,7 @@ static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, Til
         return per_thread >= 8 ? 8 : per_thread >= 4 ? 4 : 2;
     };
     long long units = (long long)(T / c.TX) * T;
-    int occ = tiles_occupancy(ctx, dtype, c, maps);
-    if (occ <= 0) return c;
+    int occ = shape_residency(dtype, c);
     if (units > occ * sms && units <= 2 * occ * sms) {
         for (int tx = c.TX + 1; tx <= std::min(T, kMaxTX); ++tx) {
             if (T % tx || tx % c.TX) continue;
@@ -253,8 +241,8 @@ static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, Til
             TileConfig w = c;
             w.TX = tx;
             w.ilp = ilp_for(w);
-            const int occ_w = tiles_occupancy(ctx, dtype, w, maps);
-            if (occ_w > 0 && (long long)(T / tx) * T <= occ_w * sms) {
+            const int occ_w = shape_residency(dtype, w);
+            if ((long long)(T / tx) * T <= occ_w * sms) {
                 c = w;
                 units = (long long)(T / tx) * T;
                 occ = occ_w;
@@ -272,8 +260,8 @@ static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, Til
         w.threads = c.threads * 2;
         if ((long long)NT * c.TX * LPT / w.threads < 8) break;
         w.ilp = ilp_for(w);
-        const int occ_w = tiles_occupancy(ctx, dtype, w, maps);
-        if (occ_w <= 0 || units > occ_w * sms) break;
+        const int occ_w = shape_residency(dtype, w);
+        if (units > occ_w * sms) break;
         c = w;
         occ = occ_w;
     }
@@ -298,9 +286,9 @@ cudaError_t launch_tiles(const TileArgs &p, const TileConfig &c, iqa_dtype dtype
                          int maps, int rows, cudaStream_t st)
 {
     switch (dtype) {
-    case IQA_F32: return launch_tiles_f32(p, c, maps, rows, st, nullptr);
-    case IQA_F16: return launch_tiles_f16(p, c, maps, rows, st, nullptr);
-    default: return launch_tiles_bf16(p, c, maps, rows, st, nullptr);
+    case IQA_F32: return launch_tiles_f32(p, c, maps, rows, st);
+    case IQA_F16: return launch_tiles_f16(p, c, maps, rows, st);
+    default: return launch_tiles_bf16(p, c, maps, rows, st);
     }
 }
 

@@ -114,6 +114,35 @@ template <> struct Elem<float> { static constexpr int VEC = 4; };
 template <> struct Elem<__half> { static constexpr int VEC = 8; };
 template <> struct Elem<__nv_bfloat16> { static constexpr int VEC = 8; };
 
+// 16-byte asynchronous copy to shared memory, past L1, with the same L2
+// prefetch hint.
+__device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void commit_copies()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Waits until all but the latest PENDING groups of this thread's copies landed.
+template <int PENDING> __device__ __forceinline__ void wait_copies()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+__device__ __forceinline__ uint4 ld_shared16(uint32_t src)
+{
+    uint4 r;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+                 : "r"(src)
+                 : "memory");
+    return r;
+}
+
 // Raw register form of VEC elements (VEC == full vector, or 1 = scalar path).
 template <typename T, int VEC> struct Raw { uint4 v; };
 template <typename T> struct Raw<T, 1> { uint32_t v; };
@@ -306,7 +335,98 @@ struct Kahan {
 // Streams one unit (RH rows x LPU vectors, top-left at xu / yu, row stride N)
 // and returns this thread's four sums.  Vector v = tid + j * THREADS of the
 // unit is (row v / LPU, column v % LPU); (row, column) advance incrementally.
-// ILP vectors of each image are in flight per thread before any is used.
+// ILP consecutive vectors of a thread are one batch: summed in order, folded,
+// and added with compensation to the thread's totals.
+//
+// Each thread keeps DEPTH vectors of each image in flight: it copies its own
+// vectors asynchronously into its own slots of a ring in shared memory, DEPTH
+// ahead of their use, and reads each back once its copy has landed, so the only
+// wait is for its own copies and no barrier is needed.  Bytes in flight then
+// depend neither on the batch size nor on registers: of batches of loads to
+// registers the compiler sank the 16-bit ones between their arithmetic (46
+// registers, one vector of each image in flight: N = 8192, N_T = 128 FP16 in
+// 61 us, 51 with the ring), and every batch drains the pipeline at its end.
+//   ring    shared address of this thread's first slot; a ring entry is
+//           THREADS slots of x, then THREADS slots of y
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B>
+__device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
+                                                     const T *__restrict__ yu, long long N,
+                                                     int RH, int LPU, float C1f, uint32_t ring,
+                                                     float (&acc)[4])
+{
+    constexpr uint32_t IMAGE = THREADS * 16, ENTRY = 2 * IMAGE;
+    const int tid = threadIdx.x;
+    const int n = RH * LPU > tid ? (RH * LPU - tid + THREADS - 1) / THREADS : 0;
+    const int row = tid / LPU;
+    int col = tid - row * LPU;
+    const int drow = THREADS / LPU;
+    const int dcol = THREADS - drow * LPU;
+    const long long step = (long long)drow * N + (long long)dcol * VEC;
+    const long long wrap = N - (long long)LPU * VEC;  // extra step past a row's end
+    long long off = (long long)row * N + (long long)col * VEC;
+    const auto issue = [&](uint32_t slot) {
+        copy_async16(slot, xu + off);
+        copy_async16(slot + IMAGE, yu + off);
+        off += step;
+        col += dcol;
+        if (col >= LPU) {
+            col -= LPU;
+            off += wrap;
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < DEPTH; ++i) {
+        if (i < n) issue(ring + i * ENTRY);
+        commit_copies();
+    }
+    Kahan ka, kb, kx, ky;
+    uint32_t slot = ring;
+    // one batch at a time, in groups of vectors read together
+    constexpr int GROUP = VEC == 4 && ILP >= 4 ? 4 : 2;
+    for (int j = 0; j < n; j += ILP) {
+        Sums2 p;
+        p.zero();
+#pragma unroll
+        for (int g = 0; g < ILP; g += GROUP) {
+            if (g > 0 && j + g >= n) break;
+            wait_copies<DEPTH - GROUP>();
+            Raw<T, VEC> rx[GROUP], ry[GROUP];
+#pragma unroll
+            for (int u = 0; u < GROUP; ++u) {
+                if (j + g + u < n) {
+                    rx[u].v = ld_shared16(slot + u * ENTRY);
+                    ry[u].v = ld_shared16(slot + u * ENTRY + IMAGE);
+                } else {
+                    // no such vector: zeros, which add exactly 0
+                    rx[u] = zero_raw<T, VEC>();
+                    ry[u] = zero_raw<T, VEC>();
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < GROUP; ++u)
+                vector_terms<T, VEC, DO_A, DO_B>(rx[u], ry[u], C1f, p);
+#pragma unroll
+            for (int u = 0; u < GROUP; ++u) {
+                if (j + g + u + DEPTH < n) issue(slot + u * ENTRY);
+                commit_copies();
+            }
+            slot += GROUP * ENTRY;
+            if (slot == ring + DEPTH * ENTRY) slot = ring;
+        }
+        if (DO_A) ka.add(p.a.x + p.a.y);
+        if (DO_B) kb.add(p.b.x + p.b.y);
+        kx.add(p.x.x + p.x.y);
+        ky.add(p.y.x + p.y.y);
+    }
+    acc[0] = ka.value();
+    acc[1] = kb.value();
+    acc[2] = kx.value();
+    acc[3] = ky.value();
+}
+
+// The same sums in the same order with each batch's loads to registers, ILP
+// vectors (or, VEC == 1, elements of any alignment) of each image in flight
+// before any is used.
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B>
 __device__ __forceinline__ void accumulate_unit(const T *__restrict__ xu,
                                                 const T *__restrict__ yu,

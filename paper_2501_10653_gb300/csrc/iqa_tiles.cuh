@@ -11,41 +11,21 @@
 
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "iqa_internal.h"
 
 namespace iqa {
 
 namespace cg = cooperative_groups;
 
-template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP>
-__global__ void __launch_bounds__(THREADS)
-    iqa_tiles_kernel(const TileArgs p)
+// Reduces the CTA's sums and writes its tiles; with S > 1 the CTAs of the
+// tile form one cluster, whose rank 0 combines and writes.
+template <int THREADS, bool OVERLAP>
+__device__ __forceinline__ void finish_unit(const TileArgs &p, const float (&acc)[4],
+                                            int tile_row, int tile_col0,
+                                            float (*red)[THREADS], float *part)
 {
-    __shared__ float red[4][THREADS];
-    __shared__ float part[kMaxTX * 4];
-
-    // programmatic dependent launch: let the next kernel in the stream be
-    // scheduled as this grid drains, and wait for the previous one (which may
-    // have written these images or maps) before the first access -- or, for
-    // an independent call (OVERLAP), only before the first write, so the
-    // loads stream while that kernel drains
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if constexpr (!OVERLAP) asm volatile("griddepcontrol.wait;" ::: "memory");
-
-    const int tile_col0 = blockIdx.x * p.TX;
-    const int srank = blockIdx.y % p.S;
-    const int tile_row = p.tile_row0 + blockIdx.y / p.S;
-    const long long row0 = (long long)tile_row * p.NT + (long long)srank * p.RH;
-    const long long col0 = (long long)tile_col0 * p.NT;
-    const T *xu = static_cast<const T *>(p.x) + row0 * p.N + col0;
-    const T *yu = static_cast<const T *>(p.y) + row0 * p.N + col0;
-
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    // the unit lies inside the image (checked build only)
-    if (IQA_CHECK(tile_row < p.T && row0 + p.RH <= p.N &&
-                  col0 + (long long)p.TX * p.NT <= p.N && p.LPU * VEC == p.TX * p.NT))
-        accumulate_unit<T, VEC, ILP, THREADS, DO_A, DO_B>(xu, yu, p.N, p.RH, p.LPU,
-                                                          p.C1f, acc);
     reduce_unit<THREADS>(acc, p.TX, p.LPU, p.LPT, red, part, CtaBarrier());
     if constexpr (OVERLAP) asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -75,20 +55,100 @@ __global__ void __launch_bounds__(THREADS)
     cluster.sync();
 }
 
-// Launches the kernel, or, with occ non-null, stores the number of its CTAs
-// that fit one SM at once (no launch).  An independent call (p.overlap) runs
-// the OVERLAP instantiation, which only the 16-byte vector paths have; the
-// stream-ordered kernels compile exactly as they would without it.
-template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP>
-static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st, int *occ)
+// Whether a launch streams its pixels through a ring in shared memory
+// (accumulate_unit_ring) or in batches of loads to registers
+// (accumulate_unit); both sum in the same order, bit for bit.  Measured back to
+// back, registers against ring, in us:
+//   * 16-bit storage, eight or more vectors a thread (ILP 8): ring.  N = 4096,
+//     N_T = 16 / 64 / 128 / 256: 17.9 / 18.0 / 17.8 / 27.8 against 15.0 / 15.0
+//     / 14.5 / 18.6; N = 8192: 48.9 / 60.9 / 61.1 / 57.7 against 43.3 / 50.6 /
+//     51.2 / 45.5.  With fewer vectors the ring's set-up is not repaid (N =
+//     512, N_T = 16: 3.4 against 4.4).
+//   * FP32, whose eight-vector batches the compiler does keep in flight: ring
+//     from kRingUnits units on, where every SM has several CTAs to run one after
+//     the other (N = 8192, N_T = 16 / 64 / 256: 79.4 / 80.0 / 89.2 against 77.9
+//     / 77.1 / 79.4); with fewer, registers (N = 4096, N_T = 64: 24.1 against
+//     27.8; N = 2048: 8.8 against 9.1).
+constexpr long long kRingUnits = 2048;
+
+template <int VEC> inline bool use_ring(const TileArgs &p, int ilp, int rows)
 {
-    if (occ)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            occ, iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, OVERLAP>, THREADS, 0);
+    if (VEC == 1 || ilp != 8) return false;
+    return VEC == 8 || (long long)(p.T / p.TX) * rows * p.S >= kRingUnits;
+}
+
+// Ring entries: 32 KB of shared memory for 128 threads (six CTAs, 192 KB in
+// flight on an SM), 64 KB for wider CTAs, which come alone or in twos or
+// threes.  Sixteen entries measured slower (N = 8192, N_T = 16 FP16: 53.7
+// against 43.3), four 1-2% slower.
+__host__ __device__ constexpr int ring_depth(int threads) { return threads == 512 ? 4 : 8; }
+
+template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP,
+          bool RING>
+__global__ void __launch_bounds__(THREADS)
+    iqa_tiles_kernel(const TileArgs p)
+{
+    extern __shared__ __align__(16) unsigned char ring[];
+    __shared__ float red[4][THREADS];
+    __shared__ float part[kMaxTX * 4];
+
+    // programmatic dependent launch: let the next kernel in the stream be
+    // scheduled as this grid drains, and wait for the previous one (which may
+    // have written these images or maps) before the first access -- or, for
+    // an independent call (OVERLAP), only before the first write, so the
+    // loads stream while that kernel drains
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (!OVERLAP) asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    const int tile_col0 = blockIdx.x * p.TX;
+    const int srank = blockIdx.y % p.S;
+    const int tile_row = p.tile_row0 + blockIdx.y / p.S;
+    const long long row0 = (long long)tile_row * p.NT + (long long)srank * p.RH;
+    const long long col0 = (long long)tile_col0 * p.NT;
+    const T *xu = static_cast<const T *>(p.x) + row0 * p.N + col0;
+    const T *yu = static_cast<const T *>(p.y) + row0 * p.N + col0;
+
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    // the unit lies inside the image (checked build only)
+    if (IQA_CHECK(tile_row < p.T && row0 + p.RH <= p.N &&
+                  col0 + (long long)p.TX * p.NT <= p.N && p.LPU * VEC == p.TX * p.NT))
+    {
+        if constexpr (RING)
+            accumulate_unit_ring<T, VEC, ILP, THREADS, ring_depth(THREADS), DO_A, DO_B>(
+                xu, yu, p.N, p.RH, p.LPU, p.C1f,
+                (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * 16, acc);
+        else
+            accumulate_unit<T, VEC, ILP, THREADS, DO_A, DO_B>(xu, yu, p.N, p.RH, p.LPU, p.C1f,
+                                                              acc);
+    }
+    finish_unit<THREADS, OVERLAP>(p, acc, tile_row, tile_col0, red, part);
+}
+
+// Launches `kern` over the units of rows x T / TX tiles, the S CTAs of a tile
+// as a cluster; `raised` holds the devices on which its dynamic shared memory
+// limit was raised to kMaxRing.
+constexpr int kMaxRing = 160 * 1024;
+
+template <typename Kernel>
+static cudaError_t launch_units(Kernel kern, std::atomic<unsigned long long> &raised,
+                                const TileArgs &p, int rows, int threads, size_t smem,
+                                cudaStream_t st)
+{
+    if (smem > 32768) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+        if (!(raised.load(std::memory_order_acquire) & bit)) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRing);
+            if (e != cudaSuccess) return e;
+            raised.fetch_or(bit, std::memory_order_release);
+        }
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.T / p.TX), (unsigned)(rows * p.S), 1);
-    cfg.blockDim = dim3(THREADS, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -102,55 +162,77 @@ static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st, int 
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
-    return cudaLaunchKernelEx(&cfg, iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, OVERLAP>,
-                              p);
+    return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-template <typename T, int VEC, int ILP, int THREADS, bool OVERLAP>
-static cudaError_t by_maps_o(const TileArgs &p, int maps, int rows, cudaStream_t st, int *occ)
+// An independent call (p.overlap) runs the OVERLAP instantiation, which only
+// the 16-byte vector paths have.
+template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP,
+          bool RING>
+static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st)
+{
+    static std::atomic<unsigned long long> raised{0};
+    return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, OVERLAP, RING>,
+                        raised, p, rows, THREADS, RING ? ring_depth(THREADS) * THREADS * 32 : 0,
+                        st);
+}
+
+template <typename T, int VEC, int ILP, int THREADS, bool OVERLAP, bool RING>
+static cudaError_t by_maps_o(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
     switch (maps) {
-    case MAPS_A: return launch_one<T, VEC, ILP, THREADS, true, false, OVERLAP>(p, rows, st, occ);
-    case MAPS_B: return launch_one<T, VEC, ILP, THREADS, false, true, OVERLAP>(p, rows, st, occ);
-    default: return launch_one<T, VEC, ILP, THREADS, true, true, OVERLAP>(p, rows, st, occ);
+    case MAPS_A:
+        return launch_one<T, VEC, ILP, THREADS, true, false, OVERLAP, RING>(p, rows, st);
+    case MAPS_B:
+        return launch_one<T, VEC, ILP, THREADS, false, true, OVERLAP, RING>(p, rows, st);
+    default: return launch_one<T, VEC, ILP, THREADS, true, true, OVERLAP, RING>(p, rows, st);
     }
 }
 
 template <typename T, int VEC, int ILP, int THREADS>
-static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t st, int *occ)
+static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
-    if (VEC > 1 && p.overlap) return by_maps_o<T, VEC, ILP, THREADS, true>(p, maps, rows, st, occ);
-    return by_maps_o<T, VEC, ILP, THREADS, false>(p, maps, rows, st, occ);
+    const bool overlap = VEC > 1 && p.overlap;
+    if constexpr (VEC > 1 && ILP == 8) {
+        if (use_ring<VEC>(p, ILP, rows))
+            return overlap ? by_maps_o<T, VEC, ILP, THREADS, true, true>(p, maps, rows, st)
+                           : by_maps_o<T, VEC, ILP, THREADS, false, true>(p, maps, rows, st);
+    }
+    if constexpr (VEC == 4 || (VEC > 1 && ILP != 8)) {
+        if (overlap) return by_maps_o<T, VEC, ILP, THREADS, true, false>(p, maps, rows, st);
+    }
+    if constexpr (VEC == 8 && ILP == 8) return cudaErrorInvalidValue;  // always the ring
+    else return by_maps_o<T, VEC, ILP, THREADS, false, false>(p, maps, rows, st);
 }
 
 template <typename T, int VEC, int ILP>
 static cudaError_t by_threads(const TileArgs &p, const TileConfig &c, int maps,
-                              int rows, cudaStream_t st, int *occ)
+                              int rows, cudaStream_t st)
 {
     switch (c.threads) {
-    case 128: return by_maps<T, VEC, ILP, 128>(p, maps, rows, st, occ);
-    case 256: return by_maps<T, VEC, ILP, 256>(p, maps, rows, st, occ);
-    case 512: return by_maps<T, VEC, ILP, 512>(p, maps, rows, st, occ);
+    case 128: return by_maps<T, VEC, ILP, 128>(p, maps, rows, st);
+    case 256: return by_maps<T, VEC, ILP, 256>(p, maps, rows, st);
+    case 512: return by_maps<T, VEC, ILP, 512>(p, maps, rows, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
 template <typename T>
 static cudaError_t launch_tiles_t(const TileArgs &p, const TileConfig &c,
-                                  int maps, int rows, cudaStream_t st, int *occ)
+                                  int maps, int rows, cudaStream_t st)
 {
     constexpr int V = Elem<T>::VEC;
     if (c.vec == 1) {
         // scalar path for unaligned images or tiles that are not a whole
         // number of 16-byte vectors wide: one launch shape only
         if (c.threads != 256 || c.ilp != 8) return cudaErrorInvalidValue;
-        return by_maps<T, 1, 8, 256>(p, maps, rows, st, occ);
+        return by_maps<T, 1, 8, 256>(p, maps, rows, st);
     }
     if (c.vec != V) return cudaErrorInvalidValue;
     switch (c.ilp) {
-    case 2: return by_threads<T, V, 2>(p, c, maps, rows, st, occ);
-    case 4: return by_threads<T, V, 4>(p, c, maps, rows, st, occ);
-    case 8: return by_threads<T, V, 8>(p, c, maps, rows, st, occ);
+    case 2: return by_threads<T, V, 2>(p, c, maps, rows, st);
+    case 4: return by_threads<T, V, 4>(p, c, maps, rows, st);
+    case 8: return by_threads<T, V, 8>(p, c, maps, rows, st);
     default: return cudaErrorInvalidValue;
     }
 }
