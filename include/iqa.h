@@ -249,6 +249,10 @@ typedef struct {
 /*
  * The launch shape the next call for this key would use with 16-byte aligned
  * inputs: the pinned (or autotuned) one if any, else the built-in heuristic.
+ * (A call without a pinned shape whose few large tiles would leave SMs idle
+ * spreads the same units over the GPU in three launches, with the same bits, and
+ * takes stream-ordered scratch of at most 256 MB for it; under a budget below
+ * that, while capturing, or without memory it runs as the shape says.)
  * Errors: IQA_ERR_INVALID_ARG.
  */
 iqa_status iqa_get_config(iqa_ctx *ctx, iqa_dtype dtype, int N, int NT, int maps,

@@ -269,14 +269,18 @@ static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, Til
 }
 
 TileConfig pick_config(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, int maps,
-                       bool aligned)
+                       bool aligned, bool *is_pinned)
 {
+    if (is_pinned) *is_pinned = false;
     {
         std::lock_guard<std::mutex> g(ctx->cfg_mu);
         auto it = ctx->pinned.find(std::make_tuple((int)dtype, N, NT, maps));
         if (it != ctx->pinned.end()) {
             const TileConfig &c = it->second;
-            if ((c.variant == 0 && c.vec == 1) || aligned) return c;
+            if ((c.variant == 0 && c.vec == 1) || aligned) {
+                if (is_pinned) *is_pinned = true;
+                return c;
+            }
         }
     }
     return fit_one_wave(ctx, N, NT, dtype, default_config(N, NT, dtype, aligned, ctx->num_sms));
@@ -322,6 +326,36 @@ TileArgs make_args(const void *x, const void *y, int N, int NT,
 
 static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
+// One pair, arguments checked: the pinned launch shape if there is one, else
+// the default one, its few large tiles split over the GPU where that pays and
+// there is scratch for it (the bits are the same).
+iqa_status run_pair(iqa_ctx *ctx, const void *x, const void *y, iqa_dtype dtype, int N, int NT,
+                    const iqa_params &P, float *lisi, float *aug, double *sums, int overlap,
+                    cudaStream_t st)
+{
+    const int maps = sums ? MAPS_AB : ((lisi ? MAPS_A : 0) | (aug ? MAPS_B : 0));
+    bool is_pinned = false;
+    const TileConfig c =
+        pick_config(ctx, N, NT, dtype, maps, aligned16(x) && aligned16(y), &is_pinned);
+    std::string why;
+    if (!any_config_valid(N, NT, dtype, c, &why)) {
+        set_error(ctx, "no launch shape for N=%d NT=%d: %s", N, NT, why.c_str());
+        return IQA_ERR_UNSUPPORTED;
+    }
+    if (c.variant == 1)
+        return run_stream_pair(ctx, x, y, dtype, N, NT, c, P, lisi, aug, sums, maps, st);
+    TileArgs a = make_args(x, y, N, NT, c, P, lisi, aug, sums);
+    a.overlap = overlap;
+    if (!is_pinned && split_pays(ctx, N, NT, dtype, c)) {
+        bool done = false;
+        const iqa_status s = run_split(ctx, a, c, dtype, maps, st, &done);
+        if (s != IQA_OK || done) return s;
+    }
+    cudaError_t e = launch_tiles(a, c, dtype, maps, N / NT, st);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
+    return IQA_OK;
+}
+
 // Shared body of iqa_lisi / iqa_auglisi / iqa_both.
 static iqa_status run_maps(iqa_ctx *ctx, const void *x, const void *y,
                            iqa_dtype dtype, int N, int NT,
@@ -346,22 +380,8 @@ static iqa_status run_maps(iqa_ctx *ctx, const void *x, const void *y,
     iqa_params P;
     s = resolve_params(ctx, params, &P);
     if (s != IQA_OK) return s;
-    const int maps = sums ? MAPS_AB : ((lisi ? MAPS_A : 0) | (aug ? MAPS_B : 0));
-    const bool aligned = aligned16(x) && aligned16(y);
-    TileConfig c = pick_config(ctx, N, NT, dtype, maps, aligned);
-    std::string why;
-    if (!any_config_valid(N, NT, dtype, c, &why)) {
-        set_error(ctx, "no launch shape for N=%d NT=%d: %s", N, NT, why.c_str());
-        return IQA_ERR_UNSUPPORTED;
-    }
-    if (c.variant == 1)
-        return run_stream_pair(ctx, x, y, dtype, N, NT, c, P, lisi, aug, sums, maps,
-                               (cudaStream_t)stream);
-    TileArgs a = make_args(x, y, N, NT, c, P, lisi, aug, sums);
-    a.overlap = ctx->independent_calls;
-    cudaError_t e = launch_tiles(a, c, dtype, maps, N / NT, (cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
-    return IQA_OK;
+    return run_pair(ctx, x, y, dtype, N, NT, P, lisi, aug, sums, ctx->independent_calls,
+                    (cudaStream_t)stream);
 }
 
 }  // namespace iqa
@@ -429,6 +449,7 @@ void iqa_destroy(iqa_ctx *ctx)
     for (cudaEvent_t ev : ctx->band_events) cudaEventDestroy(ev);
     if (ctx->ws) cudaFree(ctx->ws);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->s_copy) cudaStreamDestroy(ctx->s_copy);
     if (ctx->s_comp) cudaStreamDestroy(ctx->s_comp);
@@ -582,6 +603,9 @@ iqa_status iqa_set_option(iqa_ctx *ctx, int option, long long value)
 extern "C" unsigned int iqa_read_violations_tiles_f32();
 extern "C" unsigned int iqa_read_violations_tiles_f16();
 extern "C" unsigned int iqa_read_violations_tiles_bf16();
+extern "C" unsigned int iqa_read_violations_split_f32();
+extern "C" unsigned int iqa_read_violations_split_f16();
+extern "C" unsigned int iqa_read_violations_split_bf16();
 extern "C" unsigned int iqa_read_violations_stream_f32();
 extern "C" unsigned int iqa_read_violations_stream_f16();
 extern "C" unsigned int iqa_read_violations_stream_bf16();
@@ -597,7 +621,8 @@ iqa_status iqa_debug_violations(unsigned long long *count)
     cudaDeviceSynchronize();
     *count = (unsigned long long)iqa_read_violations_tiles_f32() +
              iqa_read_violations_tiles_f16() + iqa_read_violations_tiles_bf16() +
-             iqa_read_violations_stream_f32() + iqa_read_violations_stream_f16() +
+             iqa_read_violations_split_f32() + iqa_read_violations_split_f16() +
+             iqa_read_violations_split_bf16() + iqa_read_violations_stream_f32() + iqa_read_violations_stream_f16() +
              iqa_read_violations_stream_bf16() + iqa_read_violations_synth() +
              iqa_read_violations_merge();
     return IQA_OK;

@@ -32,6 +32,10 @@ struct iqa_ctx {
     // keyed by (dtype, N, NT, maps)
     std::mutex cfg_mu;
     std::map<std::tuple<int, int, int, int>, iqa::TileConfig> pinned;
+    // stream-ordered scratch of split tiles (iqa_split.cu)
+    std::mutex pool_mu;
+    cudaMemPool_t pool = nullptr;
+    bool pool_failed = false;
     // batched-kernel shape per dtype, set by iqa_plan_autotune
     iqa::TileConfig batch_cfg[3];
     bool has_batch_cfg[3] = {false, false, false};
@@ -62,7 +66,13 @@ bool config_valid(int N, int NT, iqa_dtype dtype, const TileConfig &c,
 TileConfig default_config(int N, int NT, iqa_dtype dtype, bool aligned,
                           int num_sms);
 TileConfig pick_config(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, int maps,
-                       bool aligned);
+                       bool aligned, bool *is_pinned = nullptr);
+bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &c);
+iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_dtype dtype,
+                     int maps, cudaStream_t st, bool *done);
+iqa_status run_pair(iqa_ctx *ctx, const void *x, const void *y, iqa_dtype dtype, int N, int NT,
+                    const iqa_params &P, float *lisi, float *aug, double *sums, int overlap,
+                    cudaStream_t st);
 cudaError_t launch_tiles(const TileArgs &p, const TileConfig &c, iqa_dtype dtype,
                          int maps, int rows, cudaStream_t st);
 struct PairDesc;

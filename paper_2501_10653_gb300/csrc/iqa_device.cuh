@@ -332,11 +332,10 @@ struct Kahan {
 };
 
 // ---------------------------------------------------------------------------
-// Streams one unit (RH rows x LPU vectors, top-left at xu / yu, row stride N)
-// and returns this thread's four sums.  Vector v = tid + j * THREADS of the
-// unit is (row v / LPU, column v % LPU); (row, column) advance incrementally.
-// ILP consecutive vectors of a thread are one batch: summed in order, folded,
-// and added with compensation to the thread's totals.
+// Sums n vectors of a unit (rows of LPU vectors, top-left at xu / yu, row
+// stride N): vectors first, first + stride, ... of its row-major order, i.e. row
+// v / LPU and column v % LPU, advanced incrementally.  ILP consecutive ones
+// are a batch: summed in order, folded, and handed to sink(A, B, Sx, Sy).
 //
 // Each thread keeps DEPTH vectors of each image in flight: it copies its own
 // vectors asynchronously into its own slots of a ring in shared memory, DEPTH
@@ -348,19 +347,18 @@ struct Kahan {
 // 61 us, 51 with the ring), and every batch drains the pipeline at its end.
 //   ring    shared address of this thread's first slot; a ring entry is
 //           THREADS slots of x, then THREADS slots of y
-template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B>
-__device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
-                                                     const T *__restrict__ yu, long long N,
-                                                     int RH, int LPU, float C1f, uint32_t ring,
-                                                     float (&acc)[4])
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B,
+          typename Sink>
+__device__ __forceinline__ void sum_vectors_ring(const T *__restrict__ xu,
+                                                 const T *__restrict__ yu, long long N, int LPU,
+                                                 int first, int stride, int n, float C1f,
+                                                 uint32_t ring, Sink sink)
 {
     constexpr uint32_t IMAGE = THREADS * 16, ENTRY = 2 * IMAGE;
-    const int tid = threadIdx.x;
-    const int n = RH * LPU > tid ? (RH * LPU - tid + THREADS - 1) / THREADS : 0;
-    const int row = tid / LPU;
-    int col = tid - row * LPU;
-    const int drow = THREADS / LPU;
-    const int dcol = THREADS - drow * LPU;
+    const int row = first / LPU;
+    int col = first - row * LPU;
+    const int drow = stride / LPU;
+    const int dcol = stride - drow * LPU;
     const long long step = (long long)drow * N + (long long)dcol * VEC;
     const long long wrap = N - (long long)LPU * VEC;  // extra step past a row's end
     long long off = (long long)row * N + (long long)col * VEC;
@@ -379,7 +377,6 @@ __device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
         if (i < n) issue(ring + i * ENTRY);
         commit_copies();
     }
-    Kahan ka, kb, kx, ky;
     uint32_t slot = ring;
     // one batch at a time, in groups of vectors read together
     constexpr int GROUP = VEC == 4 && ILP >= 4 ? 4 : 2;
@@ -413,11 +410,35 @@ __device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
             slot += GROUP * ENTRY;
             if (slot == ring + DEPTH * ENTRY) slot = ring;
         }
-        if (DO_A) ka.add(p.a.x + p.a.y);
-        if (DO_B) kb.add(p.b.x + p.b.y);
-        kx.add(p.x.x + p.x.y);
-        ky.add(p.y.x + p.y.y);
+        sink(p.a.x + p.a.y, p.b.x + p.b.y, p.x.x + p.x.y, p.y.x + p.y.y);
     }
+}
+
+// Items of `total` that a thread takes: first, first + stride, ... < total.
+__host__ __device__ __forceinline__ int items_from(int first, int stride, int total)
+{
+    return total > first ? (total - first + stride - 1) / stride : 0;
+}
+
+// Streams one unit (RH rows x LPU vectors) through the ring and returns this
+// thread's four sums: vectors tid, tid + THREADS, ..., each batch added with
+// compensation to the thread's totals.
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B>
+__device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
+                                                     const T *__restrict__ yu, long long N,
+                                                     int RH, int LPU, float C1f, uint32_t ring,
+                                                     float (&acc)[4])
+{
+    const int tid = threadIdx.x;
+    Kahan ka, kb, kx, ky;
+    sum_vectors_ring<T, VEC, ILP, THREADS, DEPTH, DO_A, DO_B>(
+        xu, yu, N, LPU, tid, THREADS, items_from(tid, THREADS, RH * LPU), C1f, ring,
+        [&](float a, float b, float x, float y) {
+            if (DO_A) ka.add(a);
+            if (DO_B) kb.add(b);
+            kx.add(x);
+            ky.add(y);
+        });
     acc[0] = ka.value();
     acc[1] = kb.value();
     acc[2] = kx.value();

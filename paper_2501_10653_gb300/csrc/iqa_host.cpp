@@ -160,21 +160,8 @@ extern "C" iqa_status iqa_both_host_many(iqa_ctx *ctx, const iqa_host_pair *pair
         if (e == cudaSuccess) e = cudaEventRecord(loaded[slot], ctx->s_copy);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->s_comp, loaded[slot], 0);
         if (e != cudaSuccess) break;
-        const int maps = dsm ? MAPS_AB : ((dl ? MAPS_A : 0) | (da ? MAPS_B : 0));
-        TileConfig c = pick_config(ctx, p.N, p.NT, dtype, maps, true);
-        std::string why;
-        if (!any_config_valid(p.N, p.NT, dtype, c, &why)) {
-            set_error(ctx, "no launch shape for N=%d NT=%d: %s", p.N, p.NT, why.c_str());
-            s = IQA_ERR_UNSUPPORTED;
-            break;
-        }
-        if (c.variant == 1) {
-            s = run_stream_pair(ctx, base, base + L.off_y, dtype, p.N, p.NT, c, P, dl, da,
-                                dsm, maps, ctx->s_comp);
-        } else {
-            TileArgs a = make_args(base, base + L.off_y, p.N, p.NT, c, P, dl, da, dsm);
-            e = launch_tiles(a, c, dtype, maps, p.N / p.NT, ctx->s_comp);
-        }
+        s = run_pair(ctx, base, base + L.off_y, dtype, p.N, p.NT, P, dl, da, dsm, 0,
+                     ctx->s_comp);
         // maps go to page-locked staging (copied out after the last pair)
         if (e == cudaSuccess && s == IQA_OK && p.lisi_map)
             e = cudaMemcpyAsync(stage + stage_off, dl, n * 4, cudaMemcpyDeviceToHost,

@@ -41,6 +41,24 @@ cudaError_t launch_tiles_f16(const TileArgs &p, const TileConfig &c, int maps,
 cudaError_t launch_tiles_bf16(const TileArgs &p, const TileConfig &c, int maps,
                               int rows, cudaStream_t st);
 
+// Tiles split over the GPU (iqa_split.cuh).
+constexpr int kSplitThreads = 128;  // threads of a CTA: a slice of a unit's
+constexpr int kSplitDepth = 8;      // ring entries
+
+struct SplitArgs {
+    TileArgs t;      // the units of iqa_tiles_kernel: S per tile, TX = 1
+    int TH;          // threads of a unit
+    int NB;          // batches of a unit
+    int PB, pieces;  // batches of a CTA, CTAs per slice of a unit
+    int maps;        // MapsMask: sums formed
+    float *parts;    // [unit][batch][sum][thread] batch sums
+    float *warps;    // [unit][sum][warp] totals
+};
+
+cudaError_t launch_split_sums_f32(const SplitArgs &p, int vec, int maps, cudaStream_t st);
+cudaError_t launch_split_sums_f16(const SplitArgs &p, int vec, int maps, cudaStream_t st);
+cudaError_t launch_split_sums_bf16(const SplitArgs &p, int vec, int maps, cudaStream_t st);
+
 struct StreamParams;
 cudaError_t launch_stream_f32(const StreamParams &sp, int ct, int maps, int grid,
                               size_t smem, cudaStream_t st);

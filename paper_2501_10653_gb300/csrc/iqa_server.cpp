@@ -428,18 +428,10 @@ iqa_status launch_step(iqa_server *srv, Slot &s)
             e = launch_synth((int)srv->cfg.dtype, s.d_jobs, s.d_synth_hdr, srv->synth_grid, s.st);
         if (e == cudaSuccess && marks) e = cudaEventRecord(s.mark[1], s.st);
         if (e == cudaSuccess) {
-            TileConfig c = pick_config(ctx, r.N, r.r.NT, srv->cfg.dtype, MAPS_AB, true);
-            if (c.variant == 1) {
-                iqa_status st = run_stream_pair(ctx, ref.d_image, pool + r.pool_off,
-                                                srv->cfg.dtype, r.N, r.r.NT, c, srv->P,
-                                                s.d_out, s.d_out + (size_t)r.T * r.T, nullptr,
-                                                MAPS_AB, s.st);
-                if (st != IQA_OK) return st;
-            } else {
-                TileArgs a = make_args(ref.d_image, pool + r.pool_off, r.N, r.r.NT, c, srv->P,
-                                       s.d_out, s.d_out + (size_t)r.T * r.T, nullptr);
-                e = launch_tiles(a, c, srv->cfg.dtype, MAPS_AB, r.T, s.st);
-            }
+            const iqa_status st =
+                run_pair(ctx, ref.d_image, pool + r.pool_off, srv->cfg.dtype, r.N, r.r.NT,
+                         srv->P, s.d_out, s.d_out + (size_t)r.T * r.T, nullptr, 0, s.st);
+            if (st != IQA_OK) return st;
         }
         if (e == cudaSuccess && marks) e = cudaEventRecord(s.mark[2], s.st);
     } else {

@@ -1,0 +1,223 @@
+// iqa_split.cu -- split tiles: the chains over the batch sums, the end of a
+// tile, and the host side (iqa_split.cuh says how the work is divided).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <mutex>
+
+#include "iqa.h"
+#include "iqa_ctx.h"
+#include "iqa_split.cuh"
+
+namespace iqa {
+
+// blockIdx.y = unit, blockIdx.x = sum * (TH / kSplitThreads) + slice: a GPU
+// thread per thread of the unit adds its batches of one sum in order, and the
+// warp's totals go through the tree of reduce_unit.  Bound by the chain, about
+// 16 cycles a batch (N = N_T = 4096 FP32: 128 batches, 1 us), as long as its
+// loads arrive in time: AHEAD of them are on their way while the previous AHEAD
+// are added.  Eight at a time, waited for each time, left the whole N = N_T =
+// 4096 call at 51.5 us (32.7 with 32 ahead); units of few batches take 8, whose
+// registers let more CTAs run at once (N = 4096, N_T = 1024: 30.6 against 40.4).
+template <int AHEAD>
+__global__ void __launch_bounds__(kSplitThreads) iqa_split_chain_kernel(const SplitArgs p)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int slices = p.TH / kSplitThreads;
+    const int q = blockIdx.x / slices, slice = blockIdx.x - q * slices;
+    if ((q == 0 && !(p.maps & MAPS_A)) || (q == 1 && !(p.maps & MAPS_B))) return;
+    const int tid = slice * kSplitThreads + threadIdx.x;
+    const int lc = blockIdx.y;
+    const int items = p.t.RH * p.t.LPU;
+    const int nb = (items_from(tid, p.TH, items) + kSplitIlp - 1) / kSplitIlp;
+    const float *in = p.parts + ((long long)lc * p.NB * 4 + q) * p.TH + tid;
+    const long long step = 4LL * p.TH;
+    Kahan k;
+    float v[2][AHEAD];
+    const auto load = [&](int b, float (&to)[AHEAD]) {
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+            if (b + i < nb) to[i] = __ldcg(in + (b + i) * step);
+    };
+    const auto add = [&](int b, const float (&from)[AHEAD]) {
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+            if (b + i < nb) k.add(from[i]);
+    };
+    load(0, v[0]);
+    for (int b = 0; b < nb; b += 2 * AHEAD) {
+        load(b + AHEAD, v[1]);
+        add(b, v[0]);
+        load(b + 2 * AHEAD, v[0]);
+        add(b + AHEAD, v[1]);
+    }
+    const float s = warp_sum(k.value());
+    if ((tid & 31) == 0) p.warps[((long long)lc * 4 + q) * (p.TH / 32) + tid / 32] = s;
+}
+
+// A warp per tile.
+__global__ void __launch_bounds__(32) iqa_split_tile_kernel(const SplitArgs p)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int tile = blockIdx.x, lane = threadIdx.x;
+    const int warps = p.TH / 32;
+    // all loads first: one latency, not one per unit
+    float v[kMaxCluster][4];
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool formed = (q != 0 || (p.maps & MAPS_A)) && (q != 1 || (p.maps & MAPS_B));
+            const float *w = p.warps + (((long long)tile * p.t.S + r) * 4 + q) * warps;
+            v[r][q] = formed && r < p.t.S && lane < warps ? __ldcg(w + lane) : 0.0f;
+        }
+    }
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r) {
+        if (r < p.t.S) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] += warp_sum(v[r][q]);
+        }
+    }
+    if (lane != 0) return;
+    combine_tile(p.t.lisi, p.t.aug, tile, s[0], s[1], s[2], s[3], p.t.C2f, p.t.Cf, p.t.Df,
+                 p.t.Cd);
+    if (p.t.sums) {
+        for (int q = 0; q < 4; ++q) p.t.sums[4LL * tile + q] = s[q];
+    }
+}
+
+namespace {
+
+template <typename Kernel>
+cudaError_t launch_after(Kernel kern, const SplitArgs &p, dim3 grid, int threads, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+// Scratch of one call, from the context's stream-ordered pool, which keeps at
+// most kScratchMost bytes between calls and is given back with the context.
+// nullptr where there is none: above kScratchMost or the context's budget,
+// while the stream is being captured (the replays of a graph may overlap, and
+// each would need scratch of its own), or out of memory.
+constexpr size_t kScratchMost = 256u << 20;
+
+float *scratch_alloc(iqa_ctx *ctx, size_t bytes, cudaStream_t st)
+{
+    if (bytes > kScratchMost || (ctx->budget && ctx->budget < kScratchMost)) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    {
+        std::lock_guard<std::mutex> g(ctx->pool_mu);
+        if (!ctx->pool && !ctx->pool_failed) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = ctx->device;
+            unsigned long long keep = kScratchMost;
+            int no = 0;  // never makes one stream wait for another
+            if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
+                cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) !=
+                    cudaSuccess ||
+                cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolReuseAllowInternalDependencies,
+                                        &no) != cudaSuccess) {
+                cudaGetLastError();
+                ctx->pool_failed = true;
+            }
+        }
+        if (ctx->pool_failed) return nullptr;
+    }
+    void *p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, bytes, ctx->pool, st) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return static_cast<float *>(p);
+}
+
+}  // namespace
+
+// Whether the units of shape c (one-pair kernel) leave so many SMs idle for so
+// long that three launches are faster.  Measured back to back, one-pair kernel
+// against split, in us:
+//   * element order (256 threads, 4 or 2 bytes a load): from 16K pixels a unit
+//     (N = 401, one tile: 58 against 8.7; N = 700, N_T = 350: 10.6 / 9.3);
+//   * 16-bit vectors: from 64K pixels (N = 600, N_T = 600: 16.8 / 8.5; N =
+//     2500, N_T = 500: 61.6 / 24.2; below, N = 1024, N_T = 512: 7.1 / 7.8);
+//   * FP32 vectors, whose units keep more bytes in flight: from 32K pixels where
+//     rows lie multiples of 2 KB apart (N = 1024, N_T = 512: 10.8 / 8.4; N =
+//     4096, N_T = 1024: 42.1 / 30.6) or units are at most 16 (N = 800, one tile:
+//     11.1 / 7.8), else from 100K (N = 1500, N_T = 500, 50K: 10.8 / 12.7).
+// With many units (FP32 two per SM, else eight) the GPU is full without it (N =
+// 4096, N_T = 512 FP32: 25.0 / 30.6).
+bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &c)
+{
+    if (c.variant != 0 || c.TX != 1 || c.ilp != kSplitIlp || c.threads % kSplitThreads != 0)
+        return false;
+    const long long T = N / NT, units = T * T * c.S;
+    const long long unit_px = (long long)NT * NT / c.S;
+    const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
+    if (c.vec == 1) return unit_px >= 16384 && units < 8 * sms;
+    if (dtype != IQA_F32) return unit_px >= 65536 && units < 8 * sms;
+    if (unit_px < 32768 || units >= 2 * sms) return false;
+    return N % 512 == 0 || units <= 16 || unit_px >= 100000;
+}
+
+// One pair in the order of the one-pair kernel's shape c; `a` as for
+// launch_tiles.  *done is false, and nothing was launched, without scratch.
+iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_dtype dtype,
+                     int maps, cudaStream_t st, bool *done)
+{
+    *done = false;
+    SplitArgs p;
+    p.t = a;
+    p.maps = maps;
+    p.TH = c.threads;
+    const long long units = (long long)a.T * a.T * a.S;
+    const long long items = (long long)a.RH * a.LPU;
+    const long long batch = (long long)p.TH * kSplitIlp;
+    const long long NB = (items + batch - 1) / batch;
+    if (items > 0x7fffffffLL - batch) return IQA_OK;
+    p.NB = (int)NB;
+    // about two waves of the six CTAs that an SM holds
+    const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
+    const long long slices = units * (p.TH / kSplitThreads);
+    const long long pieces = std::min(NB, std::max(1LL, (12 * sms + slices - 1) / slices));
+    p.PB = (int)((NB + pieces - 1) / pieces);
+    p.pieces = (int)((NB + p.PB - 1) / p.PB);
+    const size_t n_parts = (size_t)units * NB * 4 * p.TH, n_warps = (size_t)units * 4 * (p.TH / 32);
+    p.parts = scratch_alloc(ctx, (n_parts + n_warps) * sizeof(float), st);
+    if (!p.parts) return IQA_OK;
+    p.warps = p.parts + n_parts;
+    cudaError_t e = dtype == IQA_F32   ? launch_split_sums_f32(p, c.vec, maps, st)
+                    : dtype == IQA_F16 ? launch_split_sums_f16(p, c.vec, maps, st)
+                                       : launch_split_sums_bf16(p, c.vec, maps, st);
+    if (e == cudaSuccess)
+        e = launch_after(p.NB > 32 ? iqa_split_chain_kernel<32> : iqa_split_chain_kernel<8>, p,
+                         dim3((unsigned)(4 * (p.TH / kSplitThreads)), (unsigned)units),
+                         kSplitThreads, st);
+    if (e == cudaSuccess)
+        e = launch_after(iqa_split_tile_kernel, p, dim3((unsigned)(a.T * a.T)), 32, st);
+    const cudaError_t ef = cudaFreeAsync(p.parts, st);
+    if (e == cudaSuccess) e = ef;
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
+    *done = true;
+    return IQA_OK;
+}
+
+}  // namespace iqa
