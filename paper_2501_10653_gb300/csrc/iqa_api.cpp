@@ -311,6 +311,9 @@ TileArgs make_args(const void *x, const void *y, int N, int NT,
     a.RH = NT / c.S;
     a.LPT = NT / c.vec;
     a.LPU = c.TX * a.LPT;
+    a.drow = c.threads / a.LPU;
+    a.dcol = c.threads % a.LPU;
+    a.inv_lpu = 1.0f / (float)a.LPU;
     a.tile_row0 = 0;
     a.C1f = (float)P.C1;
     a.C2f = (float)P.C2;

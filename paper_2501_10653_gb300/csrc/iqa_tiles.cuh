@@ -55,20 +55,20 @@ __device__ __forceinline__ void finish_unit(const TileArgs &p, const float (&acc
     cluster.sync();
 }
 
-// Whether a launch streams its pixels through a ring in shared memory
-// (accumulate_unit_ring) or in batches of loads to registers
+// Whether a launch of vector units streams its pixels through a ring in shared
+// memory (accumulate_unit_ring) or in batches of loads to registers
 // (accumulate_unit); both sum in the same order, bit for bit.  Measured back to
 // back, registers against ring, in us:
 //   * 16-bit storage, eight or more vectors a thread (ILP 8): ring.  N = 4096,
-//     N_T = 16 / 64 / 128 / 256: 17.9 / 18.0 / 17.8 / 27.8 against 15.0 / 15.0
-//     / 14.5 / 18.6; N = 8192: 48.9 / 60.9 / 61.1 / 57.7 against 43.3 / 50.6 /
-//     51.2 / 45.5.  With fewer vectors the ring's set-up is not repaid (N =
+//     N_T = 16 / 64 / 128 / 256: 17.9 / 18.0 / 17.8 / 27.8 against 14.7 / 15.0
+//     / 14.5 / 14.2; N = 8192: 48.9 / 60.9 / 61.1 / 57.7 against 44.8 / 44.2 /
+//     44.3 / 47.7.  With fewer vectors the ring's set-up is not repaid (N =
 //     512, N_T = 16: 3.4 against 4.4).
-//   * FP32, whose eight-vector batches the compiler does keep in flight: ring
-//     from kRingUnits units on, where every SM has several CTAs to run one after
-//     the other (N = 8192, N_T = 16 / 64 / 256: 79.4 / 80.0 / 89.2 against 77.9
-//     / 77.1 / 79.4); with fewer, registers (N = 4096, N_T = 64: 24.1 against
-//     27.8; N = 2048: 8.8 against 9.1).
+//   * FP32, whose eight-vector batches the compiler keeps in flight: ring from
+//     kRingUnits units on, where every SM has several CTAs to run one after the
+//     other (N = 8192, N_T = 16 / 64 / 256: 83.6 / 79.3 / 87.5 against 77.0 /
+//     75.7 / 77.7; N = 4096, N_T = 16: 25.1 / 22.7); with fewer, registers (N =
+//     4096, N_T = 64: 22.2 against 22.8; N = 2048: 8.1 against 9.1).
 constexpr long long kRingUnits = 2048;
 
 template <int VEC> inline bool use_ring(const TileArgs &p, int ilp, int rows)
@@ -83,9 +83,29 @@ template <int VEC> inline bool use_ring(const TileArgs &p, int ilp, int rows)
 // against 43.3), four 1-2% slower.
 __host__ __device__ constexpr int ring_depth(int threads) { return threads == 512 ? 4 : 8; }
 
+// Resident CTAs to compile for.  Left to itself the compiler aims at a residency
+// of its own and sinks loads between their arithmetic for it (40 to 96
+// registers); stated, it keeps a batch in flight.  Measured back to back, in us,
+// without and with:
+//   * FP32 registers, one CTA (114 registers): N = 2048, N_T = 16 / 64 / 128 /
+//     256 8.7 / 8.9 / 8.0 / 9.4 and 8.0 / 8.1 / 7.6 / 8.6; N = 4096, N_T = 64
+//     24.2 and 22.7;
+//   * element order, four (56): N = 8001, N_T = 63 BF16 136 and 92; N = 3000, N_T =
+//     75 FP32 19.4 and 15.3 (two or three: the same; five: 16.7);
+//   * 16-bit ring, one (102): N = 2048, N_T = 128 7.2 and 5.6; N = 8192, N_T = 64
+//     49.0 and 44.2;
+//   * FP32 ring, as many as its shared memory lets in: N = 8192, N_T = 64 / 256 76.9
+//     / 79.2 and 75.8 / 77.2 (one CTA: 78.2 / 85.6).
+template <int VEC, bool STREAMED> constexpr int min_ctas(int threads)
+{
+    if (VEC == 1) return 4;
+    if (VEC == 8 || !STREAMED) return 1;
+    return threads == 128 ? 6 : threads == 256 ? 3 : 2;
+}
+
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP,
-          bool RING>
-__global__ void __launch_bounds__(THREADS)
+          bool STREAMED>
+__global__ void __launch_bounds__(THREADS, (min_ctas<VEC, STREAMED>(THREADS)))
     iqa_tiles_kernel(const TileArgs p)
 {
     extern __shared__ __align__(16) unsigned char ring[];
@@ -101,8 +121,10 @@ __global__ void __launch_bounds__(THREADS)
     if constexpr (!OVERLAP) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const int tile_col0 = blockIdx.x * p.TX;
-    const int srank = blockIdx.y % p.S;
-    const int tile_row = p.tile_row0 + blockIdx.y / p.S;
+    // (small element-order units notice the two divisions, vector units do not)
+    const int tile_row_s = VEC == 1 && p.S == 1 ? blockIdx.y : blockIdx.y / p.S;
+    const int srank = VEC == 1 && p.S == 1 ? 0 : blockIdx.y % p.S;
+    const int tile_row = p.tile_row0 + tile_row_s;
     const long long row0 = (long long)tile_row * p.NT + (long long)srank * p.RH;
     const long long col0 = (long long)tile_col0 * p.NT;
     const T *xu = static_cast<const T *>(p.x) + row0 * p.N + col0;
@@ -113,13 +135,17 @@ __global__ void __launch_bounds__(THREADS)
     if (IQA_CHECK(tile_row < p.T && row0 + p.RH <= p.N &&
                   col0 + (long long)p.TX * p.NT <= p.N && p.LPU * VEC == p.TX * p.NT))
     {
-        if constexpr (RING)
+        if constexpr (VEC > 1 && STREAMED)
             accumulate_unit_ring<T, VEC, ILP, THREADS, ring_depth(THREADS), DO_A, DO_B>(
                 xu, yu, p.N, p.RH, p.LPU, p.C1f,
                 (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * 16, acc);
+        else if constexpr (STREAMED)
+            accumulate_elements<T, ILP, THREADS, DO_A, DO_B>(xu, yu, (int)p.N, p.RH, p.LPU,
+                                                             p.drow, p.dcol, p.inv_lpu, p.C1f,
+                                                             acc);
         else
-            accumulate_unit<T, VEC, ILP, THREADS, DO_A, DO_B>(xu, yu, p.N, p.RH, p.LPU, p.C1f,
-                                                              acc);
+            accumulate_unit<T, VEC, ILP, THREADS, DO_A, DO_B>(
+                xu, yu, p.N, p.RH, p.LPU, p.drow, p.dcol, p.inv_lpu, p.C1f, acc);
     }
     finish_unit<THREADS, OVERLAP>(p, acc, tile_row, tile_col0, red, part);
 }
@@ -168,24 +194,24 @@ static cudaError_t launch_units(Kernel kern, std::atomic<unsigned long long> &ra
 // An independent call (p.overlap) runs the OVERLAP instantiation, which only
 // the 16-byte vector paths have.
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP,
-          bool RING>
+          bool STREAMED>
 static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st)
 {
     static std::atomic<unsigned long long> raised{0};
-    return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, OVERLAP, RING>,
-                        raised, p, rows, THREADS, RING ? ring_depth(THREADS) * THREADS * 32 : 0,
-                        st);
+    constexpr int smem = VEC > 1 && STREAMED ? ring_depth(THREADS) * THREADS * 32 : 0;
+    return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, OVERLAP, STREAMED>,
+                        raised, p, rows, THREADS, smem, st);
 }
 
-template <typename T, int VEC, int ILP, int THREADS, bool OVERLAP, bool RING>
+template <typename T, int VEC, int ILP, int THREADS, bool OVERLAP, bool STREAMED>
 static cudaError_t by_maps_o(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
     switch (maps) {
     case MAPS_A:
-        return launch_one<T, VEC, ILP, THREADS, true, false, OVERLAP, RING>(p, rows, st);
+        return launch_one<T, VEC, ILP, THREADS, true, false, OVERLAP, STREAMED>(p, rows, st);
     case MAPS_B:
-        return launch_one<T, VEC, ILP, THREADS, false, true, OVERLAP, RING>(p, rows, st);
-    default: return launch_one<T, VEC, ILP, THREADS, true, true, OVERLAP, RING>(p, rows, st);
+        return launch_one<T, VEC, ILP, THREADS, false, true, OVERLAP, STREAMED>(p, rows, st);
+    default: return launch_one<T, VEC, ILP, THREADS, true, true, OVERLAP, STREAMED>(p, rows, st);
     }
 }
 
@@ -197,6 +223,11 @@ static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t s
         if (use_ring<VEC>(p, ILP, rows))
             return overlap ? by_maps_o<T, VEC, ILP, THREADS, true, true>(p, maps, rows, st)
                            : by_maps_o<T, VEC, ILP, THREADS, false, true>(p, maps, rows, st);
+    }
+    if constexpr (VEC == 1) {
+        // 32-bit offsets wherever a unit's fit
+        if ((long long)(p.RH + THREADS) * p.N < 0x7fffffffLL)
+            return by_maps_o<T, VEC, ILP, THREADS, false, true>(p, maps, rows, st);
     }
     if constexpr (VEC == 4 || (VEC > 1 && ILP != 8)) {
         if (overlap) return by_maps_o<T, VEC, ILP, THREADS, true, false>(p, maps, rows, st);
