@@ -24,8 +24,9 @@
  *     to the context's device, and that device must be current.
  *   - The map kernels use programmatic dependent launch: each may be
  *     scheduled while the previous kernel in the stream drains, and waits for
- *     it before its first memory access; each lets the next kernel start
- *     early.  A caller's own kernel that follows on the stream with
+ *     it before its first memory access (the first CTAs of a one-pair call may
+ *     ask for their pixels to be brought to L2 before, which reads nothing);
+ *     each lets the next kernel start early.  A caller's own kernel that follows on the stream with
  *     programmatic stream serialization enabled must wait for its prerequisite
  *     grid (griddepcontrol.wait) before reading the maps; any other work
  *     follows in plain stream order.

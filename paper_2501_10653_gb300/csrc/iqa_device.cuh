@@ -70,6 +70,7 @@ struct TileArgs {
     int LPT;            // vectors per tile row = NT / VEC
     int drow, dcol;     // threads / LPU, threads % LPU: a thread's step
     float inv_lpu;      // 1 / LPU
+    int prefetch_ctas;  // CTAs (in launch order) that prefetch their unit to L2
     int tile_row0;      // first tile row covered by this launch
     float C1f;          // C1 rounded to float, used in the per-pixel divide
     float C2f, Cf, Df;  // Eq. 1 / Eq. 2 constants of the per-tile combine
@@ -136,6 +137,18 @@ __device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src)
                  : "memory");
+}
+
+// Starts a copy of the whole 16-byte pieces inside [p, p + bytes) to L2.  A hint:
+// nothing is read on the SM's behalf, and L2 is where every SM's writes meet, so
+// it may precede the writes of a kernel that still runs.
+__device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
+{
+    const unsigned long long a = (unsigned long long)p;
+    const unsigned long long from = (a + 15) & ~15ull, to = (a + bytes) & ~15ull;
+    if (to > from)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(from),
+                     "r"((unsigned)(to - from)));
 }
 
 __device__ __forceinline__ void commit_copies()

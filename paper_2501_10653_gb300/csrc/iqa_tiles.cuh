@@ -103,7 +103,14 @@ template <int VEC, bool STREAMED> constexpr int min_ctas(int threads)
     return threads == 128 ? 6 : threads == 256 ? 3 : 2;
 }
 
-template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP,
+// How a launch stands to the kernel before it in the stream.
+enum Order {
+    ORDER_WAIT,      // every access after it
+    ORDER_PREFETCH,  // the same, with the first CTAs' units brought to L2 before
+    ORDER_OVERLAP    // an independent call: only writes after it
+};
+
+template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int ORDER,
           bool STREAMED>
 __global__ void __launch_bounds__(THREADS, (min_ctas<VEC, STREAMED>(THREADS)))
     iqa_tiles_kernel(const TileArgs p)
@@ -115,11 +122,10 @@ __global__ void __launch_bounds__(THREADS, (min_ctas<VEC, STREAMED>(THREADS)))
     // programmatic dependent launch: let the next kernel in the stream be
     // scheduled as this grid drains, and wait for the previous one (which may
     // have written these images or maps) before the first access -- or, for
-    // an independent call (OVERLAP), only before the first write, so the
-    // loads stream while that kernel drains
+    // an independent call, only before the first write, so the loads stream
+    // while that kernel drains
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if constexpr (!OVERLAP) asm volatile("griddepcontrol.wait;" ::: "memory");
-
+    if constexpr (ORDER == ORDER_WAIT) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int tile_col0 = blockIdx.x * p.TX;
     // (small element-order units notice the two divisions, vector units do not)
     const int tile_row_s = VEC == 1 && p.S == 1 ? blockIdx.y : blockIdx.y / p.S;
@@ -129,6 +135,18 @@ __global__ void __launch_bounds__(THREADS, (min_ctas<VEC, STREAMED>(THREADS)))
     const long long col0 = (long long)tile_col0 * p.NT;
     const T *xu = static_cast<const T *>(p.x) + row0 * p.N + col0;
     const T *yu = static_cast<const T *>(p.y) + row0 * p.N + col0;
+
+    if constexpr (ORDER == ORDER_PREFETCH) {
+        if ((int)(blockIdx.y * gridDim.x + blockIdx.x) < p.prefetch_ctas &&
+            IQA_CHECK(tile_row < p.T && row0 + p.RH <= p.N &&
+                      col0 + (long long)p.TX * p.NT <= p.N)) {
+            for (long long r = threadIdx.x; r < p.RH; r += THREADS) {
+                prefetch_l2(xu + r * p.N, (unsigned)(p.LPU * VEC * (int)sizeof(T)));
+                prefetch_l2(yu + r * p.N, (unsigned)(p.LPU * VEC * (int)sizeof(T)));
+            }
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
 
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     // the unit lies inside the image (checked build only)
@@ -147,7 +165,7 @@ __global__ void __launch_bounds__(THREADS, (min_ctas<VEC, STREAMED>(THREADS)))
             accumulate_unit<T, VEC, ILP, THREADS, DO_A, DO_B>(
                 xu, yu, p.N, p.RH, p.LPU, p.drow, p.dcol, p.inv_lpu, p.C1f, acc);
     }
-    finish_unit<THREADS, OVERLAP>(p, acc, tile_row, tile_col0, red, part);
+    finish_unit<THREADS, ORDER == ORDER_OVERLAP>(p, acc, tile_row, tile_col0, red, part);
 }
 
 // Launches `kern` over the units of rows x T / TX tiles, the S CTAs of a tile
@@ -191,49 +209,55 @@ static cudaError_t launch_units(Kernel kern, std::atomic<unsigned long long> &ra
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-// An independent call (p.overlap) runs the OVERLAP instantiation, which only
-// the 16-byte vector paths have.
-template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, bool OVERLAP,
+// An independent call (p.overlap) runs the ORDER_OVERLAP instantiation, which
+// only the 16-byte vector paths have.
+template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int ORDER,
           bool STREAMED>
 static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st)
 {
     static std::atomic<unsigned long long> raised{0};
     constexpr int smem = VEC > 1 && STREAMED ? ring_depth(THREADS) * THREADS * 32 : 0;
-    return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, OVERLAP, STREAMED>,
+    return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, ORDER, STREAMED>,
                         raised, p, rows, THREADS, smem, st);
 }
 
-template <typename T, int VEC, int ILP, int THREADS, bool OVERLAP, bool STREAMED>
+template <typename T, int VEC, int ILP, int THREADS, int ORDER, bool STREAMED>
 static cudaError_t by_maps_o(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
     switch (maps) {
     case MAPS_A:
-        return launch_one<T, VEC, ILP, THREADS, true, false, OVERLAP, STREAMED>(p, rows, st);
+        return launch_one<T, VEC, ILP, THREADS, true, false, ORDER, STREAMED>(p, rows, st);
     case MAPS_B:
-        return launch_one<T, VEC, ILP, THREADS, false, true, OVERLAP, STREAMED>(p, rows, st);
-    default: return launch_one<T, VEC, ILP, THREADS, true, true, OVERLAP, STREAMED>(p, rows, st);
+        return launch_one<T, VEC, ILP, THREADS, false, true, ORDER, STREAMED>(p, rows, st);
+    default: return launch_one<T, VEC, ILP, THREADS, true, true, ORDER, STREAMED>(p, rows, st);
     }
+}
+
+template <typename T, int VEC, int ILP, int THREADS, bool STREAMED>
+static cudaError_t by_order(const TileArgs &p, int maps, int rows, cudaStream_t st)
+{
+    if (VEC > 1 && p.overlap)
+        return by_maps_o<T, VEC, ILP, THREADS, (VEC > 1 ? ORDER_OVERLAP : ORDER_WAIT), STREAMED>(
+            p, maps, rows, st);
+    if (p.prefetch_ctas > 0)
+        return by_maps_o<T, VEC, ILP, THREADS, ORDER_PREFETCH, STREAMED>(p, maps, rows, st);
+    return by_maps_o<T, VEC, ILP, THREADS, ORDER_WAIT, STREAMED>(p, maps, rows, st);
 }
 
 template <typename T, int VEC, int ILP, int THREADS>
 static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
-    const bool overlap = VEC > 1 && p.overlap;
     if constexpr (VEC > 1 && ILP == 8) {
         if (use_ring<VEC>(p, ILP, rows))
-            return overlap ? by_maps_o<T, VEC, ILP, THREADS, true, true>(p, maps, rows, st)
-                           : by_maps_o<T, VEC, ILP, THREADS, false, true>(p, maps, rows, st);
+            return by_order<T, VEC, ILP, THREADS, true>(p, maps, rows, st);
     }
     if constexpr (VEC == 1) {
         // 32-bit offsets wherever a unit's fit
         if ((long long)(p.RH + THREADS) * p.N < 0x7fffffffLL)
-            return by_maps_o<T, VEC, ILP, THREADS, false, true>(p, maps, rows, st);
-    }
-    if constexpr (VEC == 4 || (VEC > 1 && ILP != 8)) {
-        if (overlap) return by_maps_o<T, VEC, ILP, THREADS, true, false>(p, maps, rows, st);
+            return by_order<T, VEC, ILP, THREADS, true>(p, maps, rows, st);
     }
     if constexpr (VEC == 8 && ILP == 8) return cudaErrorInvalidValue;  // always the ring
-    else return by_maps_o<T, VEC, ILP, THREADS, false, false>(p, maps, rows, st);
+    else return by_order<T, VEC, ILP, THREADS, false>(p, maps, rows, st);
 }
 
 template <typename T, int VEC, int ILP>
