@@ -337,13 +337,15 @@ static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // from L2.  Measured back to back, in us, without and with: FP32 N = 2048, N_T =
 // 64 8.2 and 6.3 (one CTA per SM: 6.9; four: 6.7); N = 4096, N_T = 64 22.6 and 21.1
 // (40 MB: 22.4); N = 3000, N_T = 75 15.6 and 14.1; FP16 N = 4096, N_T = 64 15.1 and
-// 13.7.  None for large images, where the start weighs little and the prefetch
-// competes with the reads (N = 8192, N_T = 64 FP16 44.2 and 47.1), nor for 16-bit
-// clusters (N = 4096, N_T = 256 14.3 and 16.0).
+// 13.7.  None for small images, whose launches are apart anyway (an isolated one
+// then is 1 us slower), for large ones, where the start weighs little and the
+// prefetch competes with the reads (N = 8192, N_T = 64 FP16 44.2 and 47.1), nor for
+// 16-bit clusters (N = 4096, N_T = 256 14.3 and 16.0).
 static int prefetch_ctas(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_dtype dtype)
 {
     const long long es = elem_size(dtype);
-    if (2 * a.N * a.N * es >= 160 << 20 || (c.vec == 8 && a.S > 1)) return 0;
+    const long long bytes = 2 * a.N * a.N * es;
+    if (bytes < 8 << 20 || bytes >= 160 << 20 || (c.vec == 8 && a.S > 1)) return 0;
     const long long unit_bytes = 2 * (long long)a.RH * a.LPU * c.vec * es;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
     return (int)std::min(2 * sms, (20LL << 20) / unit_bytes);

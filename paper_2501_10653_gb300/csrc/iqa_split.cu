@@ -155,16 +155,16 @@ float *scratch_alloc(iqa_ctx *ctx, size_t bytes, cudaStream_t st)
 // Whether the units of shape c (one-pair kernel) leave so many SMs idle for so
 // long that three launches are faster.  Measured back to back, one-pair kernel
 // against split, in us:
-//   * element order (256 threads, 4 or 2 bytes a load): from 16K pixels a unit
-//     (N = 401, one tile: 58 against 8.7; N = 700, N_T = 350: 10.6 / 9.3);
+//   * element order (256 threads, 4 or 2 bytes a load): from 40K pixels a unit
+//     (N = 401, one tile: 58 against 8.7; below, N = 1287, N_T = 143: 10.6 / 12.4);
 //   * 16-bit vectors: from 64K pixels (N = 600, N_T = 600: 16.8 / 8.5; N =
 //     2500, N_T = 500: 61.6 / 24.2; below, N = 1024, N_T = 512: 7.1 / 7.8);
 //   * FP32 vectors, whose units keep more bytes in flight: from 32K pixels where
 //     rows lie multiples of 2 KB apart (N = 1024, N_T = 512: 10.8 / 8.4; N =
 //     4096, N_T = 1024: 42.1 / 30.6) or units are at most 16 (N = 800, one tile:
 //     11.1 / 7.8), else from 100K (N = 1500, N_T = 500, 50K: 10.8 / 12.7).
-// With many units (FP32 two per SM, else eight) the GPU is full without it (N =
-// 4096, N_T = 512 FP32: 25.0 / 30.6).
+// With many units (two per SM, 16-bit vectors eight) the GPU is full without it
+// (N = 4096, N_T = 512 FP32: 25.0 / 30.6; N = 4128, N_T = 129: 32.7 / 50.6).
 bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &c)
 {
     if (c.variant != 0 || c.TX != 1 || c.ilp != kSplitIlp || c.threads % kSplitThreads != 0)
@@ -172,7 +172,7 @@ bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &
     const long long T = N / NT, units = T * T * c.S;
     const long long unit_px = (long long)NT * NT / c.S;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
-    if (c.vec == 1) return unit_px >= 16384 && units < 8 * sms;
+    if (c.vec == 1) return unit_px >= 40000 && units < 2 * sms;
     if (dtype != IQA_F32) return unit_px >= 65536 && units < 8 * sms;
     if (unit_px < 32768 || units >= 2 * sms) return false;
     return N % 512 == 0 || units <= 16 || unit_px >= 100000;

@@ -84,22 +84,28 @@ template <int VEC> inline bool use_ring(const TileArgs &p, int ilp, int rows)
 __host__ __device__ constexpr int ring_depth(int threads) { return threads == 512 ? 4 : 8; }
 
 // Resident CTAs to compile for.  Left to itself the compiler aims at a residency
-// of its own and sinks loads between their arithmetic for it (40 to 96
-// registers); stated, it keeps a batch in flight.  Measured back to back, in us,
-// without and with:
-//   * FP32 registers, one CTA (114 registers): N = 2048, N_T = 16 / 64 / 128 /
-//     256 8.7 / 8.9 / 8.0 / 9.4 and 8.0 / 8.1 / 7.6 / 8.6; N = 4096, N_T = 64
-//     24.2 and 22.7;
-//   * element order, four (56): N = 8001, N_T = 63 BF16 136 and 92; N = 3000, N_T =
-//     75 FP32 19.4 and 15.3 (two or three: the same; five: 16.7);
-//   * 16-bit ring, one (102): N = 2048, N_T = 128 7.2 and 5.6; N = 8192, N_T = 64
-//     49.0 and 44.2;
+// of its own and sinks loads between their arithmetic for it; stated, it keeps a
+// batch in flight.  Measured back to back, in us:
+//   * FP32 batches of eight in registers: five CTAs of 128 threads (96
+//     registers), with which the one-wave rule of the launch shapes counts.
+//     Four (114 registers) gain where a launch still fits one wave (N = 2048, N_T
+//     = 64 8.8 and 8.1) and lose a wave where it does not (N = 4608, N_T = 64 27.5
+//     and 34.2);
+//   * shorter batches: as many CTAs as hold their registers without spills;
+//     fewer leave small units waiting (N = 3936, N_T = 16 BF16 60.7 and 69.8);
+//   * element order, four (56): N = 8001, N_T = 63 BF16 136 without and 92 with;
+//     N = 3000, N_T = 75 FP32 19.4 and 15.3 (two or three: the same; five: 16.7);
+//   * 16-bit ring, one (102): N = 2048, N_T = 128 7.2 without and 5.6 with; N = 8192,
+//     N_T = 64 49.0 and 44.2;
 //   * FP32 ring, as many as its shared memory lets in: N = 8192, N_T = 64 / 256 76.9
-//     / 79.2 and 75.8 / 77.2 (one CTA: 78.2 / 85.6).
-template <int VEC, bool STREAMED> constexpr int min_ctas(int threads)
+//     / 79.2 without and 75.8 / 77.2 with (one CTA: 78.2 / 85.6).
+template <int VEC, int ILP, bool STREAMED> constexpr int min_ctas(int threads)
 {
     if (VEC == 1) return 4;
-    if (VEC == 8 || !STREAMED) return 1;
+    if (ILP == 2) return threads == 128 ? 10 : threads == 256 ? 5 : 2;
+    if (ILP == 4) return threads == 128 ? 8 : threads == 256 ? 4 : 2;
+    if (!STREAMED) return threads == 128 ? 5 : threads == 256 ? 2 : 1;
+    if (VEC == 8) return 1;
     return threads == 128 ? 6 : threads == 256 ? 3 : 2;
 }
 
@@ -112,7 +118,7 @@ enum Order {
 
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int ORDER,
           bool STREAMED>
-__global__ void __launch_bounds__(THREADS, (min_ctas<VEC, STREAMED>(THREADS)))
+__global__ void __launch_bounds__(THREADS, (min_ctas<VEC, ILP, STREAMED>(THREADS)))
     iqa_tiles_kernel(const TileArgs p)
 {
     extern __shared__ __align__(16) unsigned char ring[];
