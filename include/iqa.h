@@ -338,8 +338,9 @@ typedef struct iqa_plan iqa_plan;
  * the plan is used.  Synchronous.  The launch shape is the one the context's
  * last iqa_plan_autotune picked for this dtype, else the default: 128
  * consumer threads, 3 CTAs per SM, 2 stages of 16 KB per image, units of 32K
- * pixel pairs for FP32 and 128K for 16-bit storage (iqa_plan_set_config sets
- * another).
+ * pixel pairs for FP32 and 128K for 16-bit storage, halved in tile rows while
+ * the units are still no more than the launch's CTAs (the same bits;
+ * iqa_plan_info has the units, iqa_plan_set_config sets another shape).
  * Errors: IQA_ERR_INVALID_ARG (bad pair, shape, dtype, constants),
  * IQA_ERR_UNSUPPORTED (a pair the TMA kernel cannot stream: unaligned images,
  * NT not a multiple of 16 bytes or above 256), IQA_ERR_NOMEM, IQA_ERR_CUDA.
@@ -387,8 +388,8 @@ iqa_status iqa_plan_set_config(iqa_plan *plan, const iqa_launch_config *cfg);
 
 /*
  * The unit that a plan of launch shape `cfg` (variant 1) streams one pair of
- * side N and tile side NT in, by the rules iqa_plan_create and
- * iqa_plan_set_config apply: *tiles_across whole tiles across (dividing
+ * side N and tile side NT in, by the rules iqa_plan_create (before any halving
+ * for a plan of few units) and iqa_plan_set_config apply: *tiles_across whole tiles across (dividing
  * N/NT), *tile_rows tile rows down (dividing N/NT), and *units units in the
  * pair's work list, (N/NT/tile_rows) * (N/NT/tiles_across), taken in
  * row-major order of their first tiles.  A host-only query: needs no GPU and

@@ -30,6 +30,7 @@ struct iqa_plan {
     unsigned long long *d_sched = nullptr;
     long long total_units = 0;
     int head_units = 1;  // units of each CTA's static first grab
+    bool shrink = false; // units may be smaller than cfg's (plan_build)
     int grid = 0;
     size_t table_bytes = 0;
     unsigned long long input_bytes = 0;
@@ -75,17 +76,45 @@ static iqa_status check_pair(iqa_ctx *ctx, const iqa_pair &p, iqa_dtype dtype, i
 // 256 KB, and 512 KB 0.4-0.6% slower.
 static long long head_bytes(iqa_dtype dtype) { return elem_size(dtype) == 2 ? 524288 : 262144; }
 
-// (Re)build the descriptor table for cfg and upload it.
-static iqa_status plan_build(iqa_plan *pl, const TileConfig &cfg)
+// Halvings of the unit size, in tile rows only (the width stays that of cfg,
+// so every tile is summed in the same order whatever else the plan holds), for
+// a plan whose units are fewer than its CTAs: as many as still give every unit a
+// CTA of its own.  A unit is a serial chain for its CTA (128K pixel pairs take
+// about 40 us), so with few of them the launch lasts as long as one.  More units
+// than CTAs measured slower in independent launches back to back, whose units
+// are all first grabs otherwise (48 pairs of N = 512, N_T = 32 FP16, 96 units of
+// 128K: 10.4 us a launch, 56 on new inputs; 192 of 64K: 10.3 and 34; 768 of 16K: 13.4).
+static int shrink_units(const iqa_plan *pl, const TileConfig &cfg)
+{
+    const long long slots =
+        (long long)(pl->ctx->num_sms > 0 ? pl->ctx->num_sms : 152) * cfg.ctas_per_sm;
+    const auto units_at = [&](int halvings) {
+        long long units = 0;
+        for (const iqa_pair &p : pl->pairs) {
+            TileConfig c = cfg;
+            stream_unit_shape(c, p.N, p.NT, pl->dtype, halvings);
+            units += pair_units(p.N, p.NT, c);
+        }
+        return units;
+    };
+    int best = 0;
+    for (int h = 1; h <= 8 && units_at(h) <= slots; ++h) best = h;
+    return best;
+}
+
+// (Re)build the descriptor table for cfg and upload it; `shrink`: cfg is the
+// built-in one, and its units may be made smaller (shrink_units).
+static iqa_status plan_build(iqa_plan *pl, const TileConfig &cfg, bool shrink = false)
 {
     iqa_ctx *ctx = pl->ctx;
     std::string why;
     const int n = (int)pl->pairs.size();
+    const int halvings = shrink ? shrink_units(pl, cfg) : 0;
     long long units = 0;
     for (int i = 0; i < n; ++i) {
         const iqa_pair &p = pl->pairs[i];
         TileConfig c = cfg;
-        stream_unit_shape(c, p.N, p.NT, pl->dtype);
+        stream_unit_shape(c, p.N, p.NT, pl->dtype, halvings);
         if (!stream_config_valid(p.N, p.NT, pl->dtype, c, &why)) {
             set_error(ctx, "pair %d (N=%d NT=%d): %s", i, p.N, p.NT, why.c_str());
             return IQA_ERR_INVALID_ARG;
@@ -99,18 +128,21 @@ static iqa_status plan_build(iqa_plan *pl, const TileConfig &cfg)
                                cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "descriptor upload");
     pl->cfg = cfg;
+    pl->shrink = shrink;
     pl->total_units = units;
     pl->grid = stream_grid(ctx, cfg, units);
     // each CTA's first grab spans about head_bytes() of each image (at most
     // 8 units), counted on the first pair's units (the largest); one unit of
-    // 16K-128K pixel pairs alone is 32-256 KB
+    // 16K-128K pixel pairs alone is 32-256 KB; no more than an even share of
+    // the units, or the CTAs past the last static grab would have nothing
     if (n > 0) {
         const PairDesc &d0 = pl->h_table[0];
         const long long unit_bytes =
             (long long)d0.RH * d0.TX * d0.NT * d0.NT * elem_size(pl->dtype);
         pl->head_units = (int)std::max<long long>(
-            1, std::min<long long>(8, head_bytes(pl->dtype) /
-                                          std::max<long long>(1, unit_bytes)));
+            1, std::min<long long>({8, units / pl->grid,
+                                    head_bytes(pl->dtype) /
+                                        std::max<long long>(1, unit_bytes)}));
     }
     return IQA_OK;
 }
@@ -263,11 +295,13 @@ iqa_status iqa_plan_create(iqa_ctx *ctx, const iqa_pair *pairs, int npairs, iqa_
         return IQA_ERR_NOMEM;
     }
     TileConfig cfg = default_batch_config(dtype);
+    bool chosen = false;
     {
         std::lock_guard<std::mutex> g(ctx->cfg_mu);
-        if (ctx->has_batch_cfg[dtype]) cfg = ctx->batch_cfg[dtype];
+        chosen = ctx->has_batch_cfg[dtype];
+        if (chosen) cfg = ctx->batch_cfg[dtype];
     }
-    s = plan_build(pl, cfg);
+    s = plan_build(pl, cfg, !chosen);
     if (s == IQA_OK && (flags & IQA_PLAN_GRAPH)) s = plan_capture(pl);
     cudaSetDevice(prev);
     if (s != IQA_OK) {
@@ -335,6 +369,7 @@ iqa_status iqa_plan_set_config(iqa_plan *plan, const iqa_launch_config *cfg)
     cudaGetDevice(&prev);
     cudaSetDevice(ctx->device);
     const TileConfig keep = plan->cfg;
+    const bool keep_shrink = plan->shrink;
     TileConfig c = keep;
     c.threads = cfg->threads;
     c.stages = cfg->stages;
@@ -351,7 +386,7 @@ iqa_status iqa_plan_set_config(iqa_plan *plan, const iqa_launch_config *cfg)
             std::lock_guard<std::mutex> g(ctx->err_mu);
             msg = ctx->last_error;
         }
-        const iqa_status r = plan_build(plan, keep);
+        const iqa_status r = plan_build(plan, keep, keep_shrink);
         if (r == IQA_OK) set_error(ctx, "%s", msg.c_str());
         else s = r;
     }
@@ -406,6 +441,7 @@ iqa_status iqa_plan_autotune(iqa_plan *plan, iqa_stream stream, int iters,
     if (!plan || iters < 1) return IQA_ERR_INVALID_ARG;
     iqa_ctx *ctx = plan->ctx;
     const TileConfig keep = plan->cfg;
+    const bool keep_shrink = plan->shrink;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -470,7 +506,7 @@ iqa_status iqa_plan_autotune(iqa_plan *plan, iqa_stream stream, int iters,
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    iqa_status s2 = plan_build(plan, s == IQA_OK ? best : keep);
+    iqa_status s2 = s == IQA_OK ? plan_build(plan, best) : plan_build(plan, keep, keep_shrink);
     if (s == IQA_OK) s = s2;
     if (s == IQA_OK && plan->exec) s = plan_capture(plan);
     if (s == IQA_OK) {

@@ -134,12 +134,13 @@ int stream_unit_rows(int N, int NT, iqa_dtype dtype, int threads, int TX, long l
 }
 
 // The unit of a batched launch: as wide as stream_tiles_across() allows, then
-// as many tile rows down as stream_unit_rows() allows, for c.unit_kpx.
-void stream_unit_shape(TileConfig &c, int N, int NT, iqa_dtype dtype)
+// as many tile rows down as stream_unit_rows() allows, for c.unit_kpx (the rows
+// for that size halved `halvings` times).
+void stream_unit_shape(TileConfig &c, int N, int NT, iqa_dtype dtype, int halvings)
 {
     const long long unit_px = (long long)c.unit_kpx * 1024;
     c.TX = stream_tiles_across(N, NT, dtype, c.threads, unit_px);
-    c.RH = stream_unit_rows(N, NT, dtype, c.threads, c.TX, unit_px);
+    c.RH = stream_unit_rows(N, NT, dtype, c.threads, c.TX, unit_px >> halvings);
 }
 
 TileConfig default_stream_config(int N, int NT, iqa_dtype dtype)
