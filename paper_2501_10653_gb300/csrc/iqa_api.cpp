@@ -335,7 +335,8 @@ static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // the kernel before it drains: at most two per SM, which find room beside that
 // kernel's CTAs, and about 20 MB in all.  The launch's first reads then come
 // from L2.  Measured back to back, in us, without and with: FP32 N = 2048, N_T =
-// 64 8.2 and 6.3 (one CTA per SM: 6.9; four: 6.7); N = 4096, N_T = 64 22.6 and 21.1
+// 64 9.1 and 7.0 (with four CTAs resident 8.2 and 6.3; one prefetching CTA per SM
+// 6.9, four 6.7); N = 2304, N_T = 64 FP16 7.9 and 6.7; N = 4096, N_T = 64 22.6 and 21.1
 // (40 MB: 22.4); N = 3000, N_T = 75 15.6 and 14.1; FP16 N = 4096, N_T = 64 15.1 and
 // 13.7.  None for small images, whose launches are apart anyway (an isolated one
 // then is 1 us slower), for large ones, where the start weighs little and the
