@@ -114,6 +114,15 @@ cudaError_t launch_after(Kernel kern, const SplitArgs &p, dim3 grid, int threads
 // each would need scratch of its own), or out of memory.
 constexpr size_t kScratchMost = 256u << 20;
 
+// Another stream may be under capture in the mode that forbids every thread
+// the calls that could wait for it, among them this stream's allocation and
+// release of scratch, which do not.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 float *scratch_alloc(iqa_ctx *ctx, size_t bytes, cudaStream_t st)
 {
     if (bytes > kScratchMost || (ctx->budget && ctx->budget < kScratchMost)) return nullptr;
@@ -201,6 +210,7 @@ iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_d
     p.PB = (int)((NB + pieces - 1) / pieces);
     p.pieces = (int)((NB + p.PB - 1) / p.PB);
     const size_t n_parts = (size_t)units * NB * 4 * p.TH, n_warps = (size_t)units * 4 * (p.TH / 32);
+    const RelaxedCapture relaxed;
     p.parts = scratch_alloc(ctx, (n_parts + n_warps) * sizeof(float), st);
     if (!p.parts) return IQA_OK;
     p.warps = p.parts + n_parts;

@@ -62,6 +62,32 @@ def test_captured_call_runs_without_scratch(contexts):
         assert np.array_equal(g.cpu().numpy().ravel(), w.ravel())
 
 
+def test_another_stream_under_capture():
+    """The first split call of a context (which makes its pool) while another
+    stream is being captured: the call runs at once, the capture is whole."""
+    import torch
+    from paper_2501_10653_gb300 import iqa
+    ctx = iqa.iqa_create(0, 0)
+    N = 1536
+    x, y = synth.paper_pair(N=N)
+    dx, dy = parity.to_device(x), parity.to_device(y)
+    maps = torch.full((2, 2), float("nan"), device="cuda")
+    sums = torch.full((2, 4), float("nan"), dtype=torch.float64, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        iqa.iqa_both(ctx, dx, dy, iqa.IQA_F32, N, N, PARAMS, maps[0, :1], maps[0, 1:],
+                     sums[0], side)
+        iqa.iqa_both(ctx, dx, dy, iqa.IQA_F32, N, N, PARAMS, maps[1, :1], maps[1, 1:],
+                     sums[1], torch.cuda.current_stream())
+    graph.replay()
+    torch.cuda.synchronize()
+    iqa.iqa_destroy(ctx)
+    assert torch.isfinite(sums).all() and torch.equal(sums[0], sums[1])
+    assert torch.isfinite(maps).all() and torch.equal(maps[0], maps[1])
+
+
 def test_two_streams_share_no_scratch(contexts):
     """Calls in flight on two streams at once, ten each: every result as alone."""
     import torch
