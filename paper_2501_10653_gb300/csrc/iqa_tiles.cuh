@@ -6,7 +6,9 @@
 // cluster along y; the S partial sums meet in distributed shared memory and
 // the cluster's rank-0 CTA writes the tile.  Launched with programmatic
 // dependent launch: every CTA waits for the previous grid in the stream before
-// its first access.  Included once per storage type.
+// its first access (the first ones of a launch may bring their pixels to L2
+// before that, and independent calls wait only before they write: Order).
+// Included once per storage type.
 #pragma once
 
 #include <cooperative_groups.h>
