@@ -73,9 +73,13 @@ __device__ __forceinline__ void finish_unit(const TileArgs &p, const float (&acc
 //     4096, N_T = 64: 22.2 against 22.8; N = 2048: 8.1 against 9.1).
 constexpr long long kRingUnits = 2048;
 
+// A unit of 2^31 vectors and more, whose items the ring counts in 32 bits (one
+// CTA for a 16-bit tile of 131072 pixels a side), takes registers, which walk
+// rows and columns: counted in 64 bits the 16-bit ring compiled to 84 registers
+// in place of 102, and N = 8192, N_T = 64 / 128 took 47.2 us in place of 44.0.
 template <int VEC> inline bool use_ring(const TileArgs &p, int ilp, int rows)
 {
-    if (VEC == 1 || ilp != 8) return false;
+    if (VEC == 1 || ilp != 8 || (long long)p.RH * p.LPU > 0x7fffffffLL - 512) return false;
     return VEC == 8 || (long long)(p.T / p.TX) * rows * p.S >= kRingUnits;
 }
 
@@ -264,7 +268,10 @@ static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t s
         if ((long long)(p.RH + THREADS) * p.N < 0x7fffffffLL)
             return by_order<T, VEC, ILP, THREADS, true>(p, maps, rows, st);
     }
-    if constexpr (VEC == 8 && ILP == 8) return cudaErrorInvalidValue;  // always the ring
+    // (16-bit: units of 2^31 vectors only, a long serial work of one CTA, for
+    // which the instantiation that waits for the kernel before it is enough)
+    if constexpr (VEC == 8 && ILP == 8)
+        return by_maps_o<T, VEC, ILP, THREADS, ORDER_WAIT, false>(p, maps, rows, st);
     else return by_order<T, VEC, ILP, THREADS, false>(p, maps, rows, st);
 }
 
