@@ -77,28 +77,35 @@ __device__ __forceinline__ void load_tile(double (&v)[4], const MergeArgs &a, in
     }
 }
 
-// n / d rounded to float32: the quotient of the rounded operands, corrected by
-// its FP64 residual n - q d (one step of iterative refinement), which leaves
-// less than 2^-46 of relative error before the last rounding.  A full FP64
-// quotient is formed where an operand or the quotient is outside the range in
-// which float32 keeps its precision (zeros, infinities and NaN among them).
-__device__ __forceinline__ float ratio(double n, double d)
+// n / d rounded to float32 in *q: the quotient of the rounded operands, corrected
+// by its FP64 residual n - q d (one step of iterative refinement), which leaves
+// less than 2^-43 of relative error before the last rounding.  False, and the
+// caller forms an FP64 quotient, where an operand or the quotient is outside the
+// range in which float32 keeps its precision (zeros, infinities and NaN among
+// them).
+__device__ __forceinline__ bool ratio(double n, double d, float *q)
 {
     const float fn = __double2float_rn(n), fd = __double2float_rn(d);
-    const float q = __fdiv_rn(fn, fd);
-    const float an = fabsf(fn), aq = fabsf(q);
-    if (an > 1e-30f && an < 1e30f && fd > 1e-30f && fd < 1e30f && aq > 1e-30f && aq < 1e30f)
-        return q + __fdividef(__double2float_rn(__fma_rn(-(double)q, d, n)), fd);
-    return (float)(n / d);
+    const float q0 = __fdiv_rn(fn, fd);
+    const float an = fabsf(fn), aq = fabsf(q0);
+    if (!(an > 1e-30f && an < 1e30f && fd > 1e-30f && fd < 1e30f && aq > 1e-30f && aq < 1e30f))
+        return false;
+    *q = q0 + __fdividef(__double2float_rn(__fma_rn(-(double)q0, d, n)), fd);
+    return true;
 }
 
 __device__ __forceinline__ void write_merged(const MergeArgs &a, long long b, const double (&t)[4])
 {
     const double A = t[0], B = t[1], Sx = t[2], Sy = t[3];
-    if (a.lisi) a.lisi[b] = ratio(a.D * A, fmax(Sx, Sy) + a.C2);
+    float q;
+    if (a.lisi) {
+        const double n = a.D * A, d = fmax(Sx, Sy) + a.C2;
+        a.lisi[b] = ratio(n, d, &q) ? q : (float)(n / d);
+    }
     if (a.aug) {
+        // 1 - B / d; where d is infinite and B is not, (d - B) / d would be NaN
         const double d = Sx + Sy + a.C;
-        a.aug[b] = ratio(d - B, d);  // 1 - B / d
+        a.aug[b] = ratio(d - B, d, &q) ? q : (float)(1.0 - B / d);
     }
     if (a.out_sums) {
         double *o = a.out_sums + 4 * b;
