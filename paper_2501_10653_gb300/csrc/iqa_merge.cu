@@ -13,7 +13,7 @@
 // time), then the 32 bytes read per tile: an FP64 instruction holds an SM's
 // pipe for about 16 cycles, whatever the number of its active lanes.  So sums
 // are formed with full warps, and the two quotients of a merged tile in float32
-// with one FP64 residual each (ratio()).  By block width m, measured back to
+// with one FP64 residual each, to the same rounding (ratio()).  By block width m, measured back to
 // back with all outputs, in us, against one thread (m <= 4), warp (m <= 90) or
 // cluster per merged tile with 64-bit index divisions and FP64 quotients:
 //   * m <= 4: a thread per merged tile, its tiles in 32-byte loads (T = 512: m =
@@ -21,7 +21,7 @@
 //     residency the compiler kept 32 registers and loads waited: m = 2 15.6);
 //   * m <= kColsMax: a thread per tile column and kColsRows rows (consecutive
 //     threads read consecutive tiles); the column sums meet in shared memory
-//     (T = 512: m = 8 7.3 / 20.5, m = 16 10.5 / 25.4, m = 32 8.2 / 17.4; T =
+//     (T = 512: m = 8 7.4 / 20.5, m = 16 10.5 / 25.4, m = 32 8.2 / 17.4; T =
 //     1024: m = 8 14.3 / 54.8);
 //   * larger blocks, up to the whole image: a cluster of kClusterCtas CTAs per
 //     merged tile whose partial sums meet in distributed shared memory (T =
@@ -77,12 +77,18 @@ __device__ __forceinline__ void load_tile(double (&v)[4], const MergeArgs &a, in
     }
 }
 
-// n / d rounded to float32 in *q: the quotient of the rounded operands, corrected
-// by its FP64 residual n - q d (one step of iterative refinement), which leaves
-// less than 2^-43 of relative error before the last rounding.  False, and the
-// caller forms an FP64 quotient, where an operand or the quotient is outside the
+// The FP64 quotient n / d rounded to float32 in *q, from the quotient of the
+// rounded operands and its FP64 residual n - q d (one step of iterative
+// refinement).  The correction c is at most 1.5 2^-23 of q (two rounded operands
+// and the division), itself off by at most 1.5 2^-22 of itself (rounded residual,
+// rounded divisor, __fdividef's 2 ulp), so q + c lies within 2^-43 of n / d, and
+// within that of its FP64 rounding.  Where q + c rounds the same over twice that
+// range, it is the float32 that the FP64 quotient rounds to.  Otherwise (once
+// in about 2^17 quotients), and where an operand or the quotient is outside the
 // range in which float32 keeps its precision (zeros, infinities and NaN among
-// them).
+// them), the result is false and the caller forms the FP64 quotient.  Without the
+// test of the range, quotients 2^-44 and less beside the middle of two floats
+// rounded to the wrong one.
 __device__ __forceinline__ bool ratio(double n, double d, float *q)
 {
     const float fn = __double2float_rn(n), fd = __double2float_rn(d);
@@ -90,8 +96,10 @@ __device__ __forceinline__ bool ratio(double n, double d, float *q)
     const float an = fabsf(fn), aq = fabsf(q0);
     if (!(an > 1e-30f && an < 1e30f && fd > 1e-30f && fd < 1e30f && aq > 1e-30f && aq < 1e30f))
         return false;
-    *q = q0 + __fdividef(__double2float_rn(__fma_rn(-(double)q0, d, n)), fd);
-    return true;
+    const float c = __fdividef(__double2float_rn(__fma_rn(-(double)q0, d, n)), fd);
+    const float e = aq * 0x1p-42f;
+    *q = __fadd_rn(q0, __fadd_rn(c, -e));
+    return *q == __fadd_rn(q0, __fadd_rn(c, e));
 }
 
 __device__ __forceinline__ void write_merged(const MergeArgs &a, long long b, const double (&t)[4])

@@ -1,7 +1,9 @@
 """The two quotients of a merged tile (needs a GPU) against the same FP64
-operations in numpy, for sums that are infinite or NaN.  One tile a block is not
-zero, so the sums are the inputs, exact: LISI has to be float32(D * A / (max(Sx,
-Sy) + C2)) bit for bit, and augLISI float32(1 - B / (Sx + Sy + C))."""
+operations in numpy: sums that are infinite or NaN, and quotients next to the
+middle between two float32 numbers, where only an FP64 quotient rounds the right
+way.  One tile a block (m = 1), so the sums are the inputs, exact: LISI has to be
+float32(D * A / (max(Sx, Sy) + C2)) bit for bit, and augLISI float32(1 - B /
+(Sx + Sy + C))."""
 import numpy as np
 import pytest
 
@@ -71,3 +73,26 @@ def test_equal_bright_pixels_whose_sum_overflows(ctx):
     torch.cuda.synchronize()
     assert torch.isinf(sums[0, 2:]).all() and float(sums[0, 1]) == 0.0
     assert float(aug[0]) == 1.0 and float(merged[0]) == 1.0
+
+
+@pytest.mark.parametrize("k", [34, 40, 44, 46, 48, 50])
+def test_quotients_beside_the_middle_of_two_floats(ctx, k):
+    """Quotients 2^-k off the middle, either side.  numpy's FP64 operations round
+    as the GPU's, and augLISI's quotient of 1/2 to 1 keeps 2^-52 of itself."""
+    T = 256
+    rng = np.random.default_rng(k)
+    n = T * T
+    mid = (rng.integers(1 << 23, 1 << 24, n) + 0.5) * 2.0 ** -24  # in [1/2, 1)
+    q = mid * (1 + rng.choice([-1.0, 1.0], n) * 2.0 ** -k)
+    d = rng.uniform(0.01, 2.0, n)
+    tiles = np.zeros((n, 4))
+    tiles[:, 0] = q * d
+    tiles[:, 1] = d * (1.0 - q)
+    tiles[:, 2] = d
+    # C2 = C = 0 and D = 1: the quotients are A / Sx and 1 - B / Sx
+    params = {"C1": 1e-6, "C2": 0.0, "C": 0.0, "D": 1.0}
+    lisi, aug = _merge(ctx, tiles, T, 1, params)
+    want_l, want_a = _want(tiles, params)
+    assert np.array_equal(lisi, want_l)
+    if k <= 48:
+        assert np.array_equal(aug, want_a)
