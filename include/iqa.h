@@ -113,8 +113,11 @@ iqa_status iqa_default_params(iqa_params *p);
 
 /*
  * Creates a context on CUDA device `device`.  hbm_budget_bytes caps the device
- * memory the context may allocate for its own workspace (0 = no cap).  On
- * success *out owns the context; free it with iqa_destroy.
+ * memory the context may allocate for its own workspace (0 = no cap): each of
+ * the host-buffer workspace, a plan's tables and a server's pool is refused above
+ * it, and scratch of one-pair calls (iqa_get_config) is taken only where it fits
+ * beside all that the context then holds.  On success *out owns the context;
+ * free it with iqa_destroy.
  * Errors: IQA_ERR_INVALID_ARG (out NULL, bad device), IQA_ERR_CUDA.
  */
 iqa_status iqa_create(iqa_ctx **out, int device, size_t hbm_budget_bytes);
@@ -252,8 +255,10 @@ typedef struct {
  * inputs: the pinned (or autotuned) one if any, else the built-in heuristic.
  * (A call without a pinned shape whose few large tiles would leave SMs idle
  * spreads the same units over the GPU in three launches, with the same bits, and
- * takes stream-ordered scratch of at most 256 MB for it; under a budget below
- * that, while capturing, or without memory it runs as the shape says.)
+ * takes stream-ordered scratch for it, at most 256 MB a call and 512 MB for all
+ * calls in flight; up to 256 MB stay reserved until iqa_destroy.  With less than
+ * 256 MB of the budget left, while capturing, or without memory it runs as the
+ * shape says.)
  * Errors: IQA_ERR_INVALID_ARG.
  */
 iqa_status iqa_get_config(iqa_ctx *ctx, iqa_dtype dtype, int N, int NT, int maps,

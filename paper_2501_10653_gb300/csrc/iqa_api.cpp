@@ -477,6 +477,8 @@ void iqa_destroy(iqa_ctx *ctx)
     if (ctx->ws) cudaFree(ctx->ws);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    for (cudaEvent_t ev : ctx->scratch_busy) cudaEventDestroy(ev);
+    for (cudaEvent_t ev : ctx->scratch_idle) cudaEventDestroy(ev);
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->s_copy) cudaStreamDestroy(ctx->s_copy);
     if (ctx->s_comp) cudaStreamDestroy(ctx->s_comp);

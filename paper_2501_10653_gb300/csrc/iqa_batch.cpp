@@ -33,6 +33,7 @@ struct iqa_plan {
     bool shrink = false; // units may be smaller than cfg's (plan_build)
     int grid = 0;
     size_t table_bytes = 0;
+    size_t charged = 0;  // device bytes counted against the context's budget
     unsigned long long input_bytes = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -284,6 +285,8 @@ iqa_status iqa_plan_create(iqa_ctx *ctx, const iqa_pair *pairs, int npairs, iqa_
         cudaSetDevice(prev);
         return IQA_ERR_NOMEM;
     }
+    charge_memory(ctx, need);
+    pl->charged = need;
     cudaError_t e = cudaMalloc(&pl->d_table, pl->table_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&pl->d_sched, 256);
     if (e == cudaSuccess) e = cudaMemset(pl->d_sched, 0, 256);
@@ -330,6 +333,7 @@ void iqa_plan_destroy(iqa_plan *plan)
     plan_drop_graph(plan);
     if (plan->d_table) cudaFree(plan->d_table);
     if (plan->d_sched) cudaFree(plan->d_sched);
+    credit_memory(plan->ctx, plan->charged);
     cudaSetDevice(prev);
     if (plan->h_table)
         ::operator delete(plan->h_table, std::align_val_t(alignof(PairDesc)));

@@ -32,10 +32,16 @@ struct iqa_ctx {
     // keyed by (dtype, N, NT, maps)
     std::mutex cfg_mu;
     std::map<std::tuple<int, int, int, int>, iqa::TileConfig> pinned;
-    // stream-ordered scratch of split tiles (iqa_split.cu)
+    // stream-ordered scratch of split tiles (iqa_split.cu), and what it shares
+    // the budget with: bytes of the workspace, plan tables, server pools and
+    // references (pool_mu guards all of it)
     std::mutex pool_mu;
     cudaMemPool_t pool = nullptr;
+    size_t pool_most = 0;  // the pool's size limit
     bool pool_failed = false;
+    size_t held = 0;
+    // under a budget: recorded behind split calls that may still run, and idle
+    std::vector<cudaEvent_t> scratch_busy, scratch_idle;
     // batched-kernel shape per dtype, set by iqa_plan_autotune
     iqa::TileConfig batch_cfg[3];
     bool has_batch_cfg[3] = {false, false, false};
@@ -67,6 +73,8 @@ TileConfig default_config(int N, int NT, iqa_dtype dtype, bool aligned,
                           int num_sms);
 TileConfig pick_config(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, int maps,
                        bool aligned, bool *is_pinned = nullptr);
+void charge_memory(iqa_ctx *ctx, size_t bytes);
+void credit_memory(iqa_ctx *ctx, size_t bytes);
 bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &c);
 iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_dtype dtype,
                      int maps, cudaStream_t st, bool *done);

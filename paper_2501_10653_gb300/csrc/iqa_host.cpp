@@ -31,11 +31,14 @@ iqa_status ensure_workspace(iqa_ctx *ctx, size_t need)
         cudaStreamSynchronize(ctx->s_copy);
         cudaStreamSynchronize(ctx->s_comp);
         cudaFree(ctx->ws);
+        credit_memory(ctx, ctx->ws_bytes);
         ctx->ws = nullptr;
         ctx->ws_bytes = 0;
     }
+    charge_memory(ctx, need);
     cudaError_t e = cudaMalloc(&ctx->ws, need);
     if (e != cudaSuccess) {
+        credit_memory(ctx, need);
         cudaGetLastError();
         set_error(ctx, "cudaMalloc of %zu bytes failed: %s", need, cudaGetErrorString(e));
         return IQA_ERR_NOMEM;

@@ -187,6 +187,7 @@ struct iqa_server {
     std::vector<Slot> slots;
     RangeAllocator pool;
     void *d_pool = nullptr;
+    size_t charged = 0;  // device bytes counted against the context's budget (mu)
 
     // statistics
     long long submitted = 0, completed = 0, failed = 0, steps = 0, step_pairs = 0;
@@ -882,8 +883,11 @@ iqa_status iqa_server_create(iqa_ctx *ctx, const iqa_server_config *cfg, iqa_ser
                       cfg->pool_bytes);
             return IQA_ERR_NOMEM;
         }
+        charge_memory(ctx, cfg->pool_bytes);
+        srv->charged = cfg->pool_bytes;
         cudaError_t e = cudaMalloc(&srv->d_pool, cfg->pool_bytes);
         if (e != cudaSuccess) {
+            credit_memory(ctx, srv->charged);
             cudaGetLastError();
             cudaSetDevice(prev);
             set_error(ctx, "pool of %zu bytes: %s", cfg->pool_bytes, cudaGetErrorString(e));
@@ -922,19 +926,24 @@ iqa_status iqa_server_add_reference(iqa_server *srv, int ref_id, const iqa_catal
     Reference ref;
     ref.N = cat->N;
     ref.nsrc = cat->nsrc;
+    size_t charged = 0;
     if (!srv->cfg.simulate) {
         int prev = 0;
         cudaGetDevice(&prev);
         cudaSetDevice(srv->device);
+        charged = (size_t)cat->N * cat->N * srv->es;
+        charge_memory(srv->ctx, charged);
         s = upload_reference(srv, ref, cat, seed);
         cudaSetDevice(prev);
         if (s != IQA_OK) {
             cudaFree(ref.d_arrays);
             cudaFree(ref.d_image);
+            credit_memory(srv->ctx, charged);
             return s;
         }
     }
     std::lock_guard<std::mutex> g(srv->mu);
+    srv->charged += charged;
     srv->refs[ref_id] = ref;
     return IQA_OK;
 }
@@ -1207,6 +1216,7 @@ void iqa_server_destroy(iqa_server *srv)
             cudaFree(kv.second.d_image);
         }
         cudaFree(srv->d_pool);
+        credit_memory(srv->ctx, srv->charged);
         cudaSetDevice(prev);
     }
     delete srv;

@@ -107,12 +107,21 @@ cudaError_t launch_after(Kernel kern, const SplitArgs &p, dim3 grid, int threads
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-// Scratch of one call, from the context's stream-ordered pool, which keeps at
-// most kScratchMost bytes between calls and is given back with the context.
-// nullptr where there is none: above kScratchMost or the context's budget,
-// while the stream is being captured (the replays of a graph may overlap, and
-// each would need scratch of its own), or out of memory.
+// Scratch of one call, from the context's stream-ordered pool, which holds at
+// most kPoolMost bytes for all streams together, keeps at most kScratchMost of
+// them between calls and is given back with the context.  Sizes are powers of
+// two, so that one stream's calls of any sizes fit the pool (their blocks add up
+// to less than twice the largest).  nullptr where there is none:
+//   * above kScratchMost, or with calls of other streams in flight that hold
+//     too much of the pool;
+//   * under a budget that leaves less than kScratchMost beside what the context
+//     holds otherwise (charge_memory);
+//   * while the stream is being captured: an allocation in a graph would belong
+//     to the graph, beyond the reach of the pool's limit and the budget;
+//   * out of memory.
 constexpr size_t kScratchMost = 256u << 20;
+constexpr size_t kPoolMost = 2 * kScratchMost;
+constexpr size_t kScratchLeast = 2u << 20;
 
 // Another stream may be under capture in the mode that forbids every thread
 // the calls that could wait for it, among them this stream's allocation and
@@ -123,43 +132,104 @@ struct RelaxedCapture {
     ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
+// ctx->pool_mu is held.
 float *scratch_alloc(iqa_ctx *ctx, size_t bytes, cudaStream_t st)
 {
-    if (bytes > kScratchMost || (ctx->budget && ctx->budget < kScratchMost)) return nullptr;
+    if (bytes > kScratchMost || ctx->pool_failed) return nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
         return nullptr;
     }
-    {
-        std::lock_guard<std::mutex> g(ctx->pool_mu);
-        if (!ctx->pool && !ctx->pool_failed) {
-            cudaMemPoolProps props = {};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = ctx->device;
-            unsigned long long keep = kScratchMost;
-            int no = 0;  // never makes one stream wait for another
-            if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
-                cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) !=
-                    cudaSuccess ||
-                cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolReuseAllowInternalDependencies,
-                                        &no) != cudaSuccess) {
-                cudaGetLastError();
-                ctx->pool_failed = true;
-            }
+    if (!ctx->pool) {
+        size_t most = kPoolMost;
+        if (ctx->budget) {
+            const size_t room = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
+            most = std::min(most, room / kScratchLeast * kScratchLeast);
+            if (most < kScratchMost) return nullptr;
         }
-        if (ctx->pool_failed) return nullptr;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        props.maxSize = most;
+        unsigned long long keep = kScratchMost;
+        int no = 0;  // never makes one stream wait for another
+        if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) !=
+                cudaSuccess ||
+            cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolReuseAllowInternalDependencies, &no) !=
+                cudaSuccess) {
+            cudaGetLastError();
+            ctx->pool_failed = true;
+            return nullptr;
+        }
+        ctx->pool_most = most;
     }
+    size_t size = kScratchLeast;
+    while (size < bytes) size *= 2;
     void *p = nullptr;
-    if (cudaMallocFromPoolAsync(&p, bytes, ctx->pool, st) != cudaSuccess) {
+    if (cudaMallocFromPoolAsync(&p, size, ctx->pool, st) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
     return static_cast<float *>(p);
 }
 
+// Releases the scratch behind the calls enqueued on st; under a budget also
+// records where they end, for charge_memory.  ctx->pool_mu is held.
+cudaError_t scratch_free(iqa_ctx *ctx, float *p, cudaStream_t st)
+{
+    const cudaError_t e = cudaFreeAsync(p, st);
+    if (e != cudaSuccess || !ctx->budget) return e;
+    std::vector<cudaEvent_t> &busy = ctx->scratch_busy, &idle = ctx->scratch_idle;
+    for (size_t i = 0; i < busy.size();) {
+        if (cudaEventQuery(busy[i]) == cudaSuccess) {
+            idle.push_back(busy[i]);
+            busy[i] = busy.back();
+            busy.pop_back();
+        } else {
+            ++i;
+        }
+    }
+    cudaGetLastError();  // of an event not reached yet
+    if (idle.empty()) {
+        cudaEvent_t ev;
+        const cudaError_t ec = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (ec != cudaSuccess) return ec;
+        idle.push_back(ev);
+    }
+    busy.push_back(idle.back());
+    idle.pop_back();
+    return cudaEventRecord(busy.back(), st);
+}
+
 }  // namespace
+
+// Counts `bytes` that the context is about to allocate against its budget.  The
+// scratch pool has to give way: where both do not fit, it is given back, once
+// the calls that use it have ended.
+void charge_memory(iqa_ctx *ctx, size_t bytes)
+{
+    std::lock_guard<std::mutex> g(ctx->pool_mu);
+    ctx->held += bytes;
+    if (!ctx->pool || !ctx->budget || ctx->held + ctx->pool_most <= ctx->budget) return;
+    const RelaxedCapture relaxed;
+    for (cudaEvent_t ev : ctx->scratch_busy) {
+        cudaEventSynchronize(ev);
+        ctx->scratch_idle.push_back(ev);
+    }
+    ctx->scratch_busy.clear();
+    cudaMemPoolDestroy(ctx->pool);
+    ctx->pool = nullptr;
+}
+
+// Bytes charged before and given back since.
+void credit_memory(iqa_ctx *ctx, size_t bytes)
+{
+    std::lock_guard<std::mutex> g(ctx->pool_mu);
+    ctx->held -= bytes;
+}
 
 // Whether the units of shape c (one-pair kernel) leave so many SMs idle for so
 // long that three launches are faster.  Measured back to back, one-pair kernel
@@ -211,8 +281,10 @@ iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_d
     p.pieces = (int)((NB + p.PB - 1) / p.PB);
     const size_t n_parts = (size_t)units * NB * 4 * p.TH, n_warps = (size_t)units * 4 * (p.TH / 32);
     const RelaxedCapture relaxed;
+    std::unique_lock<std::mutex> lock(ctx->pool_mu);
     p.parts = scratch_alloc(ctx, (n_parts + n_warps) * sizeof(float), st);
     if (!p.parts) return IQA_OK;
+    if (!ctx->budget) lock.unlock();  // nothing takes the pool away
     p.warps = p.parts + n_parts;
     cudaError_t e = dtype == IQA_F32   ? launch_split_sums_f32(p, c.vec, maps, st)
                     : dtype == IQA_F16 ? launch_split_sums_f16(p, c.vec, maps, st)
@@ -223,7 +295,7 @@ iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_d
                          kSplitThreads, st);
     if (e == cudaSuccess)
         e = launch_after(iqa_split_tile_kernel, p, dim3((unsigned)(a.T * a.T)), 32, st);
-    const cudaError_t ef = cudaFreeAsync(p.parts, st);
+    const cudaError_t ef = scratch_free(ctx, p.parts, st);
     if (e == cudaSuccess) e = ef;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
     *done = true;
