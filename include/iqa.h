@@ -659,6 +659,15 @@ typedef enum {
  */
 iqa_status iqa_debug_violations(unsigned long long *count);
 
+/*
+ * How the context's one-pair calls with the streaming-load kernel were launched
+ * so far: counts[0] as one kernel, counts[1] as one kernel whose first CTAs ask
+ * for their pixels in L2 before the previous kernel has ended, counts[2] split
+ * over the GPU in three launches.  For tests: all give the same bits.
+ * Errors: IQA_ERR_INVALID_ARG.
+ */
+iqa_status iqa_debug_routes(iqa_ctx *ctx, unsigned long long counts[3]);
+
 /* Sets a context option.  Errors: IQA_ERR_INVALID_ARG (unknown option or
  * value out of range: the timeout must be 1 us .. 60 s). */
 iqa_status iqa_set_option(iqa_ctx *ctx, int option, long long value);

@@ -375,11 +375,14 @@ iqa_status run_pair(iqa_ctx *ctx, const void *x, const void *y, iqa_dtype dtype,
     if (!is_pinned && split_pays(ctx, N, NT, dtype, c)) {
         bool done = false;
         const iqa_status s = run_split(ctx, a, c, dtype, maps, st, &done);
+        if (done) ctx->routes[2].fetch_add(1, std::memory_order_relaxed);
         if (s != IQA_OK || done) return s;
     }
-    a.prefetch_ctas = prefetch_ctas(ctx, a, c, dtype);
+    // (16-byte vector launches of independent calls read before they wait)
+    if (c.vec == 1 || !overlap) a.prefetch_ctas = prefetch_ctas(ctx, a, c, dtype);
     cudaError_t e = launch_tiles(a, c, dtype, maps, N / NT, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
+    ctx->routes[a.prefetch_ctas > 0].fetch_add(1, std::memory_order_relaxed);
     return IQA_OK;
 }
 
@@ -658,6 +661,13 @@ iqa_status iqa_debug_violations(unsigned long long *count)
 #else
     return IQA_ERR_UNSUPPORTED;
 #endif
+}
+
+iqa_status iqa_debug_routes(iqa_ctx *ctx, unsigned long long counts[3])
+{
+    if (!ctx || !counts) return IQA_ERR_INVALID_ARG;
+    for (int i = 0; i < 3; ++i) counts[i] = ctx->routes[i].load(std::memory_order_relaxed);
+    return IQA_OK;
 }
 
 iqa_status iqa_wait(iqa_ctx *ctx, iqa_stream stream, int timeout_us)

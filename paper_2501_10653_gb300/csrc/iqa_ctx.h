@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <string>
@@ -32,6 +33,8 @@ struct iqa_ctx {
     // keyed by (dtype, N, NT, maps)
     std::mutex cfg_mu;
     std::map<std::tuple<int, int, int, int>, iqa::TileConfig> pinned;
+    // one-pair calls by route, see iqa_debug_routes
+    std::atomic<unsigned long long> routes[3] = {};
     // stream-ordered scratch of split tiles (iqa_split.cu), and what it shares
     // the budget with: bytes of the workspace, plan tables, server pools and
     // references (pool_mu guards all of it)

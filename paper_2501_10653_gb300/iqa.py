@@ -166,6 +166,7 @@ def _declare(lib):
         "iqa_set_config": ([_vp, _i, _i, _i, _i, P(iqa_launch_config)], _st),
         "iqa_wait": ([_vp, _vp, _i], _st),
         "iqa_debug_violations": ([P(ctypes.c_ulonglong)], _st),
+        "iqa_debug_routes": ([_vp, P(ctypes.c_ulonglong)], _st),
         "iqa_set_option": ([_vp, _i, ctypes.c_longlong], _st),
         "iqa_plan_create": ([_vp, P(iqa_pair), _i, _i, P(iqa_params), _i, P(_vp)], _st),
         "iqa_plan_launch": ([_vp, _vp], _st),
@@ -324,6 +325,13 @@ def iqa_debug_violations():
     n = ctypes.c_ulonglong(0)
     _check(None, lib().iqa_debug_violations(ctypes.byref(n)))
     return n.value
+
+
+def iqa_debug_routes(ctx):
+    """One-pair calls so far: (one kernel, one kernel that prefetches, split)."""
+    n = (ctypes.c_ulonglong * 3)()
+    _check(ctx, lib().iqa_debug_routes(ctx, n))
+    return tuple(n)
 
 
 def iqa_wait(ctx, stream=None, timeout_us=-1):
