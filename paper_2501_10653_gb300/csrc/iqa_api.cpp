@@ -635,6 +635,7 @@ iqa_status iqa_set_option(iqa_ctx *ctx, int option, long long value)
 extern "C" unsigned int iqa_read_violations_tiles_f32();
 extern "C" unsigned int iqa_read_violations_tiles_f16();
 extern "C" unsigned int iqa_read_violations_tiles_bf16();
+extern "C" unsigned int iqa_read_violations_split();
 extern "C" unsigned int iqa_read_violations_split_f32();
 extern "C" unsigned int iqa_read_violations_split_f16();
 extern "C" unsigned int iqa_read_violations_split_bf16();
@@ -653,8 +654,9 @@ iqa_status iqa_debug_violations(unsigned long long *count)
     cudaDeviceSynchronize();
     *count = (unsigned long long)iqa_read_violations_tiles_f32() +
              iqa_read_violations_tiles_f16() + iqa_read_violations_tiles_bf16() +
-             iqa_read_violations_split_f32() + iqa_read_violations_split_f16() +
-             iqa_read_violations_split_bf16() + iqa_read_violations_stream_f32() + iqa_read_violations_stream_f16() +
+             iqa_read_violations_split() + iqa_read_violations_split_f32() +
+             iqa_read_violations_split_f16() + iqa_read_violations_split_bf16() +
+             iqa_read_violations_stream_f32() + iqa_read_violations_stream_f16() +
              iqa_read_violations_stream_bf16() + iqa_read_violations_synth() +
              iqa_read_violations_merge();
     return IQA_OK;

@@ -104,6 +104,7 @@ __device__ __forceinline__ bool ratio(double n, double d, float *q)
 
 __device__ __forceinline__ void write_merged(const MergeArgs &a, long long b, const double (&t)[4])
 {
+    if (!IQA_CHECK(b < (long long)a.M * a.M)) return;
     const double A = t[0], B = t[1], Sx = t[2], Sy = t[3];
     float q;
     if (a.lisi) {

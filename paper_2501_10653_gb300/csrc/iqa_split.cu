@@ -30,7 +30,11 @@ __global__ void __launch_bounds__(kSplitThreads) iqa_split_chain_kernel(const Sp
     const int tid = slice * kSplitThreads + threadIdx.x;
     const int lc = blockIdx.y;
     const int items = p.t.RH * p.t.LPU;
-    const int nb = (items_from(tid, p.TH, items) + kSplitIlp - 1) / kSplitIlp;
+    int nb = (items_from(tid, p.TH, items) + kSplitIlp - 1) / kSplitIlp;
+    // the unit, its threads, batches and warps have a place in the scratch
+    // (checked build only)
+    const bool warp_ok = IQA_CHECK(lc < p.t.T * p.t.T * p.t.S && q < 4 && tid < p.TH);
+    if (!IQA_CHECK(nb <= p.NB) || !warp_ok) nb = 0;
     const float *in = p.parts + ((long long)lc * p.NB * 4 + q) * p.TH + tid;
     const long long step = 4LL * p.TH;
     Kahan k;
@@ -53,7 +57,7 @@ __global__ void __launch_bounds__(kSplitThreads) iqa_split_chain_kernel(const Sp
         add(b + AHEAD, v[1]);
     }
     const float s = warp_sum(k.value());
-    if ((tid & 31) == 0) p.warps[((long long)lc * 4 + q) * (p.TH / 32) + tid / 32] = s;
+    if ((tid & 31) == 0 && warp_ok) p.warps[((long long)lc * 4 + q) * (p.TH / 32) + tid / 32] = s;
 }
 
 // A warp per tile.
@@ -63,6 +67,9 @@ __global__ void __launch_bounds__(32) iqa_split_tile_kernel(const SplitArgs p)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int tile = blockIdx.x, lane = threadIdx.x;
     const int warps = p.TH / 32;
+    // the tile has a place in the map, a unit's warps one in the warp (checked
+    // build only)
+    if (!IQA_CHECK(tile < p.t.T * p.t.T && warps <= 32 && p.t.S <= kMaxCluster)) return;
     // all loads first: one latency, not one per unit
     float v[kMaxCluster][4];
 #pragma unroll
@@ -303,3 +310,5 @@ iqa_status run_split(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_d
 }
 
 }  // namespace iqa
+
+IQA_VIOLATION_READER(iqa_read_violations_split)
