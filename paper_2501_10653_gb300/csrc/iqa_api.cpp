@@ -316,6 +316,7 @@ TileArgs make_args(const void *x, const void *y, int N, int NT,
     a.dcol = c.threads % a.LPU;
     a.inv_lpu = 1.0f / (float)a.LPU;
     a.prefetch_ctas = 0;
+    a.spread = 0;
     a.tile_row0 = 0;
     a.C1f = (float)P.C1;
     a.C2f = (float)P.C2;
@@ -352,6 +353,25 @@ static int prefetch_ctas(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, i
     return (int)std::min(2 * sms, (20LL << 20) / unit_bytes);
 }
 
+// Most CTAs that an element-order launch may have on one SM: its even share, up to
+// the three below the four that fit.  A launch whose CTAs are placed while the
+// kernel before it drains otherwise fills whichever SMs have room, with up to
+// four on one and none on others, and lasts as long as the fullest.  Back to
+// back, in us, placed freely and spread: 81 units N = 1287, N_T = 143 FP32 11.8 and
+// 6.1, N = 1089, N_T = 121 FP16 9.7 and 4.8; 324 units N = 2250, N_T = 125 FP32 12.8
+// and 10.1; 400 units N = 1800, N_T = 90 BF16 6.9 and 5.7; but 36 units N = 858,
+// N_T = 143 FP16 7.7 and 8.2, which leave room for two launches side by side.
+// Isolated launches are spread anyway.  (An SM whose last kernel had another
+// split of L1 and shared memory is reconfigured: after each of a caller's own
+// elementwise kernels the 81 units take 0.7 us more.)
+static int spread_ctas(iqa_ctx *ctx, int N, int NT, const TileConfig &c)
+{
+    if (c.vec != 1) return 0;
+    const long long T = N / NT, units = T / c.TX * T * c.S;
+    const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
+    return 4 * units > sms && units <= 3 * sms ? (int)((units + sms - 1) / sms) : 0;
+}
+
 // One pair, arguments checked: the pinned launch shape if there is one, else
 // the default one, its few large tiles split over the GPU where that pays and
 // there is scratch for it (the bits are the same).
@@ -380,6 +400,7 @@ iqa_status run_pair(iqa_ctx *ctx, const void *x, const void *y, iqa_dtype dtype,
     }
     // (16-byte vector launches of independent calls read before they wait)
     if (c.vec == 1 || !overlap) a.prefetch_ctas = prefetch_ctas(ctx, a, c, dtype);
+    a.spread = spread_ctas(ctx, N, NT, c);
     cudaError_t e = launch_tiles(a, c, dtype, maps, N / NT, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
     ctx->routes[a.prefetch_ctas > 0].fetch_add(1, std::memory_order_relaxed);

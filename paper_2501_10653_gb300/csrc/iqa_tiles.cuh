@@ -221,6 +221,13 @@ static cudaError_t launch_units(Kernel kern, std::atomic<unsigned long long> &ra
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
+// Dynamic shared memory of which at most `ctas` CTAs fit an SM's 228 KB beside
+// their static part and the 1 KB that each is charged.
+constexpr int spread_smem(int threads, int ctas)
+{
+    return 228 * 1024 / (ctas + 1) - (4 * threads + 4 * kMaxTX) * (int)sizeof(float);
+}
+
 // An independent call (p.overlap) runs the ORDER_OVERLAP instantiation, which
 // only the 16-byte vector paths have.
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int ORDER,
@@ -228,7 +235,8 @@ template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int O
 static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st)
 {
     static std::atomic<unsigned long long> raised{0};
-    constexpr int smem = VEC > 1 && STREAMED ? ring_depth(THREADS) * THREADS * 32 : 0;
+    int smem = VEC > 1 && STREAMED ? ring_depth(THREADS) * THREADS * 32 : 0;
+    if (VEC == 1 && p.spread > 0) smem = spread_smem(THREADS, p.spread);
     return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, ORDER, STREAMED>,
                         raised, p, rows, THREADS, smem, st);
 }
