@@ -239,18 +239,31 @@ void credit_memory(iqa_ctx *ctx, size_t bytes)
 }
 
 // Whether the units of shape c (one-pair kernel) leave so many SMs idle for so
-// long that three launches are faster.  Measured back to back, one-pair kernel
-// against split, in us:
-//   * element order (256 threads, 4 or 2 bytes a load): from 40K pixels a unit
-//     (N = 401, one tile: 58 against 8.7; below, N = 1287, N_T = 143: 10.6 / 12.4);
-//   * 16-bit vectors: from 64K pixels (N = 600, N_T = 600: 16.8 / 8.5; N =
-//     2500, N_T = 500: 61.6 / 24.2; below, N = 1024, N_T = 512: 7.1 / 7.8);
-//   * FP32 vectors, whose units keep more bytes in flight: from 32K pixels where
-//     rows lie multiples of 2 KB apart (N = 1024, N_T = 512: 10.8 / 8.4; N =
-//     4096, N_T = 1024: 42.1 / 30.6) or units are at most 16 (N = 800, one tile:
-//     11.1 / 7.8), else from 100K (N = 1500, N_T = 500, 50K: 10.8 / 12.7).
-// With many units (two per SM, 16-bit vectors eight) the GPU is full without it
-// (N = 4096, N_T = 512 FP32: 25.0 / 30.6; N = 4128, N_T = 129: 32.7 / 50.6).
+// long that three launches are faster.  Measured one-pair kernel against split,
+// in us, back to back / a call alone:
+//   * element order (256 threads, 4 or 2 bytes a load), which runs one CTA an SM
+//     up to 152 units (run_pair): the split takes its three launches and the
+//     image's bytes, the units the time of one.  N = 401, one tile of 161K pixels:
+//     31.3 / 45 against 8.6 / 23; tiles of N_T = 211 (45K): 9 units 13.1 / 24
+//     against 9.9 / 25, 36 18.3 / 24 and 15.0 / 28, 64 15.1 / 29 and 17.9 / 30, 144
+//     20.0 / 30 and 23.3 / 39.  So fewer units the smaller they are: 4.8M pixels
+//     and a pixel for each unit below 152.
+//   * vectors: not from one unit per SM on (FP32 N = 3072, N_T = 512, 288 units:
+//     18.5 / 26 against 20.5 / 31; N = 6200, N_T = 1240: 55.7 / 69 and 62.2 / 77; FP16
+//     N = 8192, N_T = 1024, 512 units: 42.8 / 57 and 57.3 / 68).  With a third to two
+//     thirds of a unit per SM the clusters find an SM for each CTA, and the
+//     split pays for few shapes (72 units of 131K pixels: FP32 18.7 / 30 against
+//     20.7 / 31, FP16 12.8 / 25 and 15.4 / 28; of 524K FP16 38.3 / 52 and 37.0 / 48);
+//     with two thirds to one it pays again (128 units of 131K: FP32 35.0 / 42
+//     against 30.6 / 42, FP16 24.5 / 36 and 21.1 / 33).
+//     - 16 bits: from 100K pixels (one tile N = 1024: 11.6 / 24 against 8.9 / 22;
+//       below, N = 800: 8.4 / 21 and 8.5 / 22, 4 tiles N = 1600: 9.2 / 22 and 11.5 /
+//       24).
+//     - FP32, whose units keep more bytes in flight: from 32K pixels where rows
+//       lie multiples of 2 KB apart (N = 1536, N_T = 512: 14.9 / 22 against 11.7 /
+//       23; N = 2048: 17.7 / 23 and 13.2 / 26), from 50K where units are at most 16
+//       (N = 728, one tile: 11.1 / 22 and 8.4 / 22; below, N = 600: 7.7 / 20 and 8.4 /
+//       21), else from 100K (4 tiles N = 1600, 80K: 11.0 / 24 and 11.1 / 24).
 bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &c)
 {
     if (c.variant != 0 || c.TX != 1 || c.ilp != kSplitIlp || c.threads % kSplitThreads != 0)
@@ -258,10 +271,12 @@ bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &
     const long long T = N / NT, units = T * T * c.S;
     const long long unit_px = (long long)NT * NT / c.S;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
-    if (c.vec == 1) return unit_px >= 40000 && units < 2 * sms;
-    if (dtype != IQA_F32) return unit_px >= 65536 && units < 8 * sms;
-    if (unit_px < 32768 || units >= 2 * sms) return false;
-    return N % 512 == 0 || units <= 16 || unit_px >= 100000;
+    if (units >= sms || unit_px < 32768) return false;
+    if (c.vec == 1) return unit_px >= 40000 && (sms - units) * unit_px > 4800000;
+    const bool one_an_sm = 3 * units > sms && 3 * units <= 2 * sms;
+    if (dtype != IQA_F32) return unit_px >= (one_an_sm ? 400000 : 100000);
+    if (unit_px >= 100000) return !one_an_sm;
+    return N % 512 == 0 || (units <= 16 && unit_px >= 50000);
 }
 
 // One pair in the order of the one-pair kernel's shape c; `a` as for
