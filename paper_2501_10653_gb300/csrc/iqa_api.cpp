@@ -316,7 +316,7 @@ TileArgs make_args(const void *x, const void *y, int N, int NT,
     a.dcol = c.threads % a.LPU;
     a.inv_lpu = 1.0f / (float)a.LPU;
     a.prefetch_ctas = 0;
-    a.spread = 0;
+    a.per_sm = 0;
     a.tile_row0 = 0;
     a.C1f = (float)P.C1;
     a.C2f = (float)P.C2;
@@ -339,37 +339,33 @@ static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // 64 9.1 and 7.0 (with four CTAs resident 8.2 and 6.3; one prefetching CTA per SM
 // 6.9, four 6.7); N = 2304, N_T = 64 FP16 7.9 and 6.7; N = 4096, N_T = 64 22.6 and 21.1
 // (40 MB: 22.4); N = 3000, N_T = 75 15.6 and 14.1; FP16 N = 4096, N_T = 64 15.1 and
-// 13.7.  None for small images, whose launches are apart anyway (an isolated one
-// then is 1 us slower), for large ones, where the start weighs little and the
-// prefetch competes with the reads (N = 8192, N_T = 64 FP16 44.2 and 47.1), nor for
-// 16-bit clusters (N = 4096, N_T = 256 14.3 and 16.0).
+// 13.7.  The price is 1 to 1.5 us on an isolated launch, whose other CTAs' reads wait
+// behind the prefetch (FP32 N = 1152, N_T = 64 15.5 and 16.7, against 5.0 and 3.9
+// back to back on inputs not in L2; N = 2048, N_T = 128 16.3 and 17.9, 6.5 and 5.4).
+// None for small images, whose launches are apart anyway; for large ones, where
+// the start weighs little and the prefetch competes with the reads (N = 8192, N_T =
+// 64 FP16 44.2 and 47.1); for 16-bit clusters (N = 4096, N_T = 256 14.3 and 16.0);
+// nor for 16-bit units in batches of two, a few KB in rows of 32 to 128 bytes that
+// a request each brings (N = 1536, N_T = 32 5.0 and 5.3, N = 2656, N_T = 32 12.3 and
+// 13.3, N = 4928, N_T = 32 28.3 and 31.3).
 static int prefetch_ctas(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, iqa_dtype dtype)
 {
     const long long es = elem_size(dtype);
     const long long bytes = 2 * a.N * a.N * es;
-    if (bytes < 8 << 20 || bytes >= 160 << 20 || (c.vec == 8 && a.S > 1)) return 0;
+    if (bytes < 8 << 20 || bytes >= 160 << 20) return 0;
+    if (c.vec == 8 && (a.S > 1 || c.ilp == 2)) return 0;
     const long long unit_bytes = 2 * (long long)a.RH * a.LPU * c.vec * es;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
     return (int)std::min(2 * sms, (20LL << 20) / unit_bytes);
 }
 
-// Most CTAs that an element-order launch may have on one SM: its even share, up to
-// the three below the four that fit.  A launch whose CTAs are placed while the
-// kernel before it drains otherwise fills whichever SMs have room, with up to
-// four on one and none on others, and lasts as long as the fullest.  Back to
-// back, in us, placed freely and spread: 81 units N = 1287, N_T = 143 FP32 11.8 and
-// 6.1, N = 1089, N_T = 121 FP16 9.7 and 4.8; 324 units N = 2250, N_T = 125 FP32 12.8
-// and 10.1; 400 units N = 1800, N_T = 90 BF16 6.9 and 5.7; but 36 units N = 858,
-// N_T = 143 FP16 7.7 and 8.2, which leave room for two launches side by side.
-// Isolated launches are spread anyway.  (An SM whose last kernel had another
-// split of L1 and shared memory is reconfigured: after each of a caller's own
-// elementwise kernels the 81 units take 0.7 us more.)
-static int spread_ctas(iqa_ctx *ctx, int N, int NT, const TileConfig &c)
+// The units of a one-pair launch that fall to an SM, 0 for less than a quarter.
+static int units_per_sm(iqa_ctx *ctx, int N, int NT, const TileConfig &c)
 {
-    if (c.vec != 1) return 0;
     const long long T = N / NT, units = T / c.TX * T * c.S;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
-    return 4 * units > sms && units <= 3 * sms ? (int)((units + sms - 1) / sms) : 0;
+    if (4 * units <= sms) return 0;
+    return (int)std::min<long long>((units + sms - 1) / sms, 1 << 30);
 }
 
 // One pair, arguments checked: the pinned launch shape if there is one, else
@@ -400,7 +396,7 @@ iqa_status run_pair(iqa_ctx *ctx, const void *x, const void *y, iqa_dtype dtype,
     }
     // (16-byte vector launches of independent calls read before they wait)
     if (c.vec == 1 || !overlap) a.prefetch_ctas = prefetch_ctas(ctx, a, c, dtype);
-    a.spread = spread_ctas(ctx, N, NT, c);
+    a.per_sm = units_per_sm(ctx, N, NT, c);
     cudaError_t e = launch_tiles(a, c, dtype, maps, N / NT, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tile kernel launch");
     ctx->routes[a.prefetch_ctas > 0].fetch_add(1, std::memory_order_relaxed);

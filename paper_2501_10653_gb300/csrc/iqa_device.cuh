@@ -82,7 +82,7 @@ struct TileArgs {
                         // stream writes none of these images and touches none
                         // of the outputs): wait for that kernel only before
                         // writing; 0: wait before any access
-    int spread;         // element order: most CTAs of the launch on one SM (0: any)
+    int per_sm;         // units per SM, rounded up (0: fewer than a quarter)
 };
 
 // ---------------------------------------------------------------------------

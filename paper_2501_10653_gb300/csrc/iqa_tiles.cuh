@@ -98,7 +98,12 @@ __host__ __device__ constexpr int ring_depth(int threads) { return threads == 51
 //     = 64 8.8 and 8.1) and lose a wave where it does not (N = 4608, N_T = 64 27.5
 //     and 34.2);
 //   * shorter batches: as many CTAs as hold their registers without spills;
-//     fewer leave small units waiting (N = 3936, N_T = 16 BF16 60.7 and 69.8);
+//     fewer leave small units waiting (N = 3936, N_T = 16 BF16 60.7 and 69.8).
+//     16-bit batches of two keep more in flight with fewer, so launches whose
+//     units all fit at once take eight or nine (by_maps: inputs not in L2, ten /
+//     nine / eight: N = 1536, N_T = 32 FP16, 1152 units 5.9 / 5.6 / 5.1, N = 1440,
+//     N_T = 48, 900 units 5.3 / 5.2 / 4.6, N = 1664, N_T = 32, 1352 units 6.0 / 5.7 /
+//     6.2; N = 3232, N_T = 32, 10201 units 17.3 / 18.0 / 18.8);
 //   * element order, four (56): N = 8001, N_T = 63 BF16 136 without and 92 with;
 //     N = 3000, N_T = 75 FP32 19.4 and 15.3 (two or three: the same; five: 16.7);
 //   * 16-bit ring, one (102): N = 2048, N_T = 128 7.2 without and 5.6 with; N = 8192,
@@ -123,8 +128,8 @@ enum Order {
 };
 
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int ORDER,
-          bool STREAMED>
-__global__ void __launch_bounds__(THREADS, (min_ctas<VEC, ILP, STREAMED>(THREADS)))
+          bool STREAMED, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS)
     iqa_tiles_kernel(const TileArgs p)
 {
     extern __shared__ __align__(16) unsigned char ring[];
@@ -221,8 +226,20 @@ static cudaError_t launch_units(Kernel kern, std::atomic<unsigned long long> &ra
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-// Dynamic shared memory of which at most `ctas` CTAs fit an SM's 228 KB beside
-// their static part and the 1 KB that each is charged.
+// Element-order launches of up to three units per SM are spread: they ask for as
+// much dynamic shared memory as lets an SM's 228 KB hold `ctas` CTAs, their even
+// share, beside the static part and the 1 KB that each is charged.  A launch
+// whose CTAs are placed while the kernel before it drains otherwise fills
+// whichever SMs have room, with up to four CTAs on one and none on others, and
+// lasts as long as the fullest.  Back to back, in us, placed freely and spread: 81
+// units N = 1287, N_T = 143 FP32 11.8 and 6.1, N = 1089, N_T = 121 FP16 9.7 and 4.8;
+// 324 units N = 2250, N_T = 125 FP32 12.8 and 10.1; 400 units N = 1800, N_T = 90 BF16
+// 6.9 and 5.7; but 36 units N = 858, N_T = 143 FP16 7.7 and 8.2, which leave room
+// for two launches side by side.  Isolated launches are spread anyway.  (An SM
+// whose last kernel had another split of L1 and shared memory is reconfigured:
+// after each of a caller's own elementwise kernels the 81 units take 0.7 us more.)
+constexpr int kSpreadMost = 3;
+
 constexpr int spread_smem(int threads, int ctas)
 {
     return 228 * 1024 / (ctas + 1) - (4 * threads + 4 * kMaxTX) * (int)sizeof(float);
@@ -231,37 +248,46 @@ constexpr int spread_smem(int threads, int ctas)
 // An independent call (p.overlap) runs the ORDER_OVERLAP instantiation, which
 // only the 16-byte vector paths have.
 template <typename T, int VEC, int ILP, int THREADS, bool DO_A, bool DO_B, int ORDER,
-          bool STREAMED>
+          bool STREAMED, int CTAS>
 static cudaError_t launch_one(const TileArgs &p, int rows, cudaStream_t st)
 {
     static std::atomic<unsigned long long> raised{0};
     int smem = VEC > 1 && STREAMED ? ring_depth(THREADS) * THREADS * 32 : 0;
-    if (VEC == 1 && p.spread > 0) smem = spread_smem(THREADS, p.spread);
-    return launch_units(iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, ORDER, STREAMED>,
-                        raised, p, rows, THREADS, smem, st);
+    if (VEC == 1 && p.per_sm >= 1 && p.per_sm <= kSpreadMost)
+        smem = spread_smem(THREADS, p.per_sm);
+    return launch_units(
+        iqa_tiles_kernel<T, VEC, ILP, THREADS, DO_A, DO_B, ORDER, STREAMED, CTAS>, raised, p, rows,
+        THREADS, smem, st);
 }
 
-template <typename T, int VEC, int ILP, int THREADS, int ORDER, bool STREAMED>
+template <typename T, int VEC, int ILP, int THREADS, int ORDER, bool STREAMED,
+          int CTAS = min_ctas<VEC, ILP, STREAMED>(THREADS)>
 static cudaError_t by_maps_o(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
     switch (maps) {
     case MAPS_A:
-        return launch_one<T, VEC, ILP, THREADS, true, false, ORDER, STREAMED>(p, rows, st);
+        return launch_one<T, VEC, ILP, THREADS, true, false, ORDER, STREAMED, CTAS>(p, rows, st);
     case MAPS_B:
-        return launch_one<T, VEC, ILP, THREADS, false, true, ORDER, STREAMED>(p, rows, st);
-    default: return launch_one<T, VEC, ILP, THREADS, true, true, ORDER, STREAMED>(p, rows, st);
+        return launch_one<T, VEC, ILP, THREADS, false, true, ORDER, STREAMED, CTAS>(p, rows, st);
+    default:
+        return launch_one<T, VEC, ILP, THREADS, true, true, ORDER, STREAMED, CTAS>(p, rows, st);
     }
 }
 
-template <typename T, int VEC, int ILP, int THREADS, bool STREAMED>
+template <typename T, int VEC, int ILP, int THREADS, bool STREAMED,
+          int CTAS = min_ctas<VEC, ILP, STREAMED>(THREADS)>
 static cudaError_t by_order(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
     if (VEC > 1 && p.overlap)
-        return by_maps_o<T, VEC, ILP, THREADS, (VEC > 1 ? ORDER_OVERLAP : ORDER_WAIT), STREAMED>(
-            p, maps, rows, st);
-    if (p.prefetch_ctas > 0)
-        return by_maps_o<T, VEC, ILP, THREADS, ORDER_PREFETCH, STREAMED>(p, maps, rows, st);
-    return by_maps_o<T, VEC, ILP, THREADS, ORDER_WAIT, STREAMED>(p, maps, rows, st);
+        return by_maps_o<T, VEC, ILP, THREADS, (VEC > 1 ? ORDER_OVERLAP : ORDER_WAIT), STREAMED,
+                         CTAS>(p, maps, rows, st);
+    // (16-bit batches of two never prefetch)
+    if constexpr (VEC != 8 || ILP != 2) {
+        if (p.prefetch_ctas > 0)
+            return by_maps_o<T, VEC, ILP, THREADS, ORDER_PREFETCH, STREAMED, CTAS>(p, maps, rows,
+                                                                                  st);
+    }
+    return by_maps_o<T, VEC, ILP, THREADS, ORDER_WAIT, STREAMED, CTAS>(p, maps, rows, st);
 }
 
 template <typename T, int VEC, int ILP, int THREADS>
@@ -270,6 +296,10 @@ static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t s
     if constexpr (VEC > 1 && ILP == 8) {
         if (use_ring<VEC>(p, ILP, rows))
             return by_order<T, VEC, ILP, THREADS, true>(p, maps, rows, st);
+    }
+    if constexpr (VEC == 8 && ILP == 2 && THREADS == 128) {
+        if (p.per_sm <= 8) return by_order<T, VEC, ILP, THREADS, false, 8>(p, maps, rows, st);
+        if (p.per_sm == 9) return by_order<T, VEC, ILP, THREADS, false, 9>(p, maps, rows, st);
     }
     if constexpr (VEC == 1) {
         // 32-bit offsets wherever a unit's fit
