@@ -106,8 +106,18 @@ __host__ __device__ constexpr int ring_depth(int threads) { return threads == 51
 //     6.2; N = 3232, N_T = 32, 10201 units 17.3 / 18.0 / 18.8);
 //   * element order, four (56): N = 8001, N_T = 63 BF16 136 without and 92 with;
 //     N = 3000, N_T = 75 FP32 19.4 and 15.3 (two or three: the same; five: 16.7);
-//   * 16-bit ring, one (102): N = 2048, N_T = 128 7.2 without and 5.6 with; N = 8192,
-//     N_T = 64 49.0 and 44.2;
+//   * 16-bit ring, one (102, so four CTAs of 128 threads): N = 2048, N_T = 128 7.2
+//     without and 5.6 with; N = 8192, N_T = 64 49.0 and 44.2.  That suits long units.
+//     With few vectors a thread a CTA's start and end weigh more, and six (72
+//     registers, as many as the shared memory lets in) cover them: from six units
+//     per SM on, with fewer than 16 vectors always (four and six: N = 3456, N_T =
+//     64 BF16 12.4 and 10.9, N = 5504 26.8 and 22.6; with five per SM N = 2400, N_T =
+//     96 7.2 and 8.1), with fewer than 32 but for seven to nine per SM, which make
+//     a second, nearly empty wave of six (N = 3840, N_T = 64 BF16, six 12.9 and
+//     10.7; N = 4864, ten 20.2 and 17.3; but N = 4096, N_T = 128 FP16, seven 12.8 and
+//     13.2).  A CTA of 512 threads has an SM to itself; two (64 registers) where
+//     that leaves a second wave (N = 4368, N_T = 728 FP16 24.7 and 17.1; N = 4800,
+//     N_T = 800 BF16 27.3 and 19.4);
 //   * FP32 ring, as many as its shared memory lets in: N = 8192, N_T = 64 / 256 76.9
 //     / 79.2 without and 75.8 / 77.2 with (one CTA: 78.2 / 85.6).
 template <int VEC, int ILP, bool STREAMED> constexpr int min_ctas(int threads)
@@ -294,8 +304,18 @@ template <typename T, int VEC, int ILP, int THREADS>
 static cudaError_t by_maps(const TileArgs &p, int maps, int rows, cudaStream_t st)
 {
     if constexpr (VEC > 1 && ILP == 8) {
-        if (use_ring<VEC>(p, ILP, rows))
+        if (use_ring<VEC>(p, ILP, rows)) {
+            if constexpr (VEC == 8 && THREADS == 128) {
+                const int vectors = p.RH * p.LPU / THREADS;  // a thread's
+                const bool waves = p.per_sm == 6 || p.per_sm > 9;
+                if (p.S == 1 && p.per_sm > 5 && (vectors < 16 || (vectors < 32 && waves)))
+                    return by_order<T, VEC, ILP, THREADS, true, 6>(p, maps, rows, st);
+            }
+            if constexpr (VEC == 8 && THREADS == 512) {
+                if (p.per_sm > 1) return by_order<T, VEC, ILP, THREADS, true, 2>(p, maps, rows, st);
+            }
             return by_order<T, VEC, ILP, THREADS, true>(p, maps, rows, st);
+        }
     }
     if constexpr (VEC == 8 && ILP == 2 && THREADS == 128) {
         if (p.per_sm <= 8) return by_order<T, VEC, ILP, THREADS, false, 8>(p, maps, rows, st);

@@ -45,3 +45,12 @@ def _check(ctx, orc, N, NT, dt, ilp):
 @pytest.mark.parametrize("N,NT", [(256, 16), (1536, 32), (1600, 32), (1664, 32), (1376, 32)])
 def test_batches_of_two(ctx, orc, dt, N, NT):
     _check(ctx, orc, N, NT, dt, 2)
+
+
+# the ring: 8 to 9 vectors a thread with 625, 722 and 882 units (five and six per
+# SM), 16 with 900 and 1024 (six and seven); 512 threads with 128 and 200
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+@pytest.mark.parametrize("N,NT", [(2400, 96), (2432, 64), (2688, 64), (3840, 64), (4096, 128),
+                                  (2912, 728), (3640, 728)])
+def test_ring(ctx, orc, dt, N, NT):
+    _check(ctx, orc, N, NT, dt, 8)
