@@ -343,9 +343,10 @@ typedef struct iqa_plan iqa_plan;
  * the plan is used.  Synchronous.  The launch shape is the one the context's
  * last iqa_plan_autotune picked for this dtype, else the default: 128
  * consumer threads, 3 CTAs per SM, 2 stages of 16 KB per image, units of 32K
- * pixel pairs for FP32 and 128K for 16-bit storage, halved in tile rows while
- * the units are still no more than the launch's CTAs (the same bits;
- * iqa_plan_info has the units, iqa_plan_set_config sets another shape).
+ * pixel pairs for FP32 and 128K for 16-bit storage.  Units of either are halved
+ * in tile rows while they are still no more than the launch's CTAs (the same
+ * bits; iqa_plan_info has the units; iqa_plan_set_config sets another shape and
+ * leaves its units as they are, as does tuning the plan itself).
  * Errors: IQA_ERR_INVALID_ARG (bad pair, shape, dtype, constants),
  * IQA_ERR_UNSUPPORTED (a pair the TMA kernel cannot stream: unaligned images,
  * NT not a multiple of 16 bytes or above 256), IQA_ERR_NOMEM, IQA_ERR_CUDA.

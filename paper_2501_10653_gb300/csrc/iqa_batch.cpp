@@ -104,7 +104,8 @@ static int shrink_units(const iqa_plan *pl, const TileConfig &cfg)
 }
 
 // (Re)build the descriptor table for cfg and upload it; `shrink`: cfg is the
-// built-in one, and its units may be made smaller (shrink_units).
+// built-in one or was tuned on another plan, and its units may be made smaller
+// (shrink_units).  A shape set by hand, or tuned on this plan, stays as it is.
 static iqa_status plan_build(iqa_plan *pl, const TileConfig &cfg, bool shrink = false)
 {
     iqa_ctx *ctx = pl->ctx;
@@ -298,13 +299,11 @@ iqa_status iqa_plan_create(iqa_ctx *ctx, const iqa_pair *pairs, int npairs, iqa_
         return IQA_ERR_NOMEM;
     }
     TileConfig cfg = default_batch_config(dtype);
-    bool chosen = false;
     {
         std::lock_guard<std::mutex> g(ctx->cfg_mu);
-        chosen = ctx->has_batch_cfg[dtype];
-        if (chosen) cfg = ctx->batch_cfg[dtype];
+        if (ctx->has_batch_cfg[dtype]) cfg = ctx->batch_cfg[dtype];
     }
-    s = plan_build(pl, cfg, !chosen);
+    s = plan_build(pl, cfg, true);
     if (s == IQA_OK && (flags & IQA_PLAN_GRAPH)) s = plan_capture(pl);
     cudaSetDevice(prev);
     if (s != IQA_OK) {

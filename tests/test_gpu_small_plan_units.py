@@ -22,6 +22,30 @@ CASES = [
 ]
 
 
+def test_units_of_a_tuned_context(ctx):  # noqa: F811
+    """A shape tuned on a large plan serves a later plan of one small pair, whose
+    units are halved all the same: 16 of one tile row, whatever the unit size of
+    the tuned shape (4K to 128K pixel pairs), with the bits of that shape set by
+    hand."""
+    import torch
+    from paper_2501_10653_gb300 import iqa
+    own = iqa.iqa_create(0, 0)
+    large = Batch([(1024, 64)] * 24, seed=63)
+    plan = iqa.iqa_plan_create(own, large.pairs(), iqa.IQA_F32, None, 0)
+    tuned = iqa.iqa_plan_autotune(plan, torch.cuda.current_stream(), 3)
+    assert iqa.iqa_plan_info(plan).config.unit_kpx == tuned.unit_kpx
+    iqa.iqa_plan_destroy(plan)
+    small = Batch([(256, 16)], seed=64)
+    info = _run(own, small)
+    got = small.results(0)
+    assert info.config.unit_kpx == tuned.unit_kpx and info.config.threads == tuned.threads
+    assert info.total_units == 16
+    _plan_with_shape(own, small, tuned)
+    for u, v in zip(got, small.results(0)):
+        assert np.array_equal(u, v)
+    iqa.iqa_destroy(own)
+
+
 @pytest.mark.parametrize("specs,dt,plain_units,units", CASES)
 def test_units(ctx, specs, dt, plain_units, units):  # noqa: F811
     from paper_2501_10653_gb300 import iqa
