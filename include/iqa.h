@@ -344,9 +344,10 @@ typedef struct iqa_plan iqa_plan;
  * last iqa_plan_autotune picked for this dtype, else the default: 128
  * consumer threads, 3 CTAs per SM, 2 stages of 16 KB per image, units of 32K
  * pixel pairs for FP32 and 128K for 16-bit storage.  Units of either are halved
- * in tile rows while they are still no more than the launch's CTAs (the same
- * bits; iqa_plan_info has the units; iqa_plan_set_config sets another shape and
- * leaves its units as they are, as does tuning the plan itself).
+ * in tile rows while they are still no more than the launch's CTAs, half of them
+ * for an independent plan (the same bits; iqa_plan_info has the units;
+ * iqa_plan_set_config sets another shape and leaves its units as they are, as
+ * does tuning the plan itself).
  * Errors: IQA_ERR_INVALID_ARG (bad pair, shape, dtype, constants),
  * IQA_ERR_UNSUPPORTED (a pair the TMA kernel cannot stream: unaligned images,
  * NT not a multiple of 16 bytes or above 256), IQA_ERR_NOMEM, IQA_ERR_CUDA.

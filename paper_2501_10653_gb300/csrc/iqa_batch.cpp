@@ -81,14 +81,22 @@ static long long head_bytes(iqa_dtype dtype) { return elem_size(dtype) == 2 ? 52
 // so every tile is summed in the same order whatever else the plan holds), for
 // a plan whose units are fewer than its CTAs: as many as still give every unit a
 // CTA of its own.  A unit is a serial chain for its CTA (128K pixel pairs take
-// about 40 us), so with few of them the launch lasts as long as one.  More units
-// than CTAs measured slower in independent launches back to back, whose units
-// are all first grabs otherwise (48 pairs of N = 512, N_T = 32 FP16, 96 units of
-// 128K: 10.4 us a launch, 56 on new inputs; 192 of 64K: 10.3 and 34; 768 of 16K: 13.4).
+// about 30 us), so with few of them the launch lasts as long as one.  Launches of
+// an independent plan overlap, each with the CTAs that the last one leaves, and
+// smaller units cost them more than they save: as many halvings as leave half
+// of the CTAs to the next launch.  Measured in us, back to back with inputs not
+// in L2 / a launch alone, by units:
+//   * graph replays of 48 pairs of N = 512, N_T = 32 FP16: 96 units of 128K 26.7 /
+//     35, 192 22.6 / 31, 384 20.6 / 29, 768 22.8 / 32; of 8 pairs 16 units 23.1 / 32,
+//     128 10.3 / 20;
+//   * the same as independent launches: 96 units 7.8 / 37, 192 8.6 / 32, 384 10.6 /
+//     32, 768 13.5 / 32; of 24 pairs 48 units 4.6 / 35, 96 4.4 / 27, 192 5.2 / 26,
+//     384 7.3 / 25; of 8 pairs 16 units 3.3 / 33, 128 3.6 / 20.
 static int shrink_units(const iqa_plan *pl, const TileConfig &cfg)
 {
-    const long long slots =
+    long long slots =
         (long long)(pl->ctx->num_sms > 0 ? pl->ctx->num_sms : 152) * cfg.ctas_per_sm;
+    if (pl->flags & IQA_PLAN_INDEPENDENT) slots /= 2;
     const auto units_at = [&](int halvings) {
         long long units = 0;
         for (const iqa_pair &p : pl->pairs) {

@@ -1,7 +1,7 @@
 """How many units a plan of few units has (needs a GPU): halved in tile rows while
-they are no more than the launch's 456 CTAs (three on each of 152 SMs), as the
-host-only geometry query counts them, and the bits of the plan whose shape is set
-by hand, which keeps its units."""
+they are no more than the launch's 456 CTAs (three on each of 152 SMs; half of
+them for an independent plan), as the host-only geometry query counts them, and
+the bits of the plan whose shape is set by hand, which keeps its units."""
 import numpy as np
 import pytest
 
@@ -9,16 +9,17 @@ from test_gpu_batch import Batch, _plan_with_shape, _run, ctx  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
-# (pairs, dtype, units of the shape as it is, units of the plan): rows halved to
-# one; halved until more would be too many; one tile row a unit already; more
-# units than CTAs already
+# (pairs, dtype, units of the shape as it is, of the plan, of an independent plan):
+# rows halved to one; halved until more would be too many; one tile row a unit
+# already; more units than CTAs already
 CASES = [
-    ([(256, 16)], "f32", 2, 16),
-    ([(1024, 16), (512, 32)], "f32", 40, 144),
-    ([(512, 32)] * 9, "bf16", 18, 144),
-    ([(512, 32)] * 48, "f16", 96, 384),
-    ([(512, 64)] * 3, "f32", 24, 24),
-    ([(1024, 16)] * 15, "f32", 480, 480),
+    ([(256, 16)], "f32", 2, 16, 16),
+    ([(1024, 16), (512, 32)], "f32", 40, 144, 144),
+    ([(512, 32)] * 9, "bf16", 18, 144, 144),
+    ([(512, 32)] * 48, "f16", 96, 384, 192),
+    ([(1024, 16)] * 5, "f32", 160, 320, 160),
+    ([(512, 64)] * 3, "f32", 24, 24, 24),
+    ([(1024, 16)] * 15, "f32", 480, 480, 480),
 ]
 
 
@@ -46,18 +47,20 @@ def test_units_of_a_tuned_context(ctx):  # noqa: F811
     iqa.iqa_destroy(own)
 
 
-@pytest.mark.parametrize("specs,dt,plain_units,units", CASES)
-def test_units(ctx, specs, dt, plain_units, units):  # noqa: F811
+@pytest.mark.parametrize("specs,dt,plain_units,units,units_independent", CASES)
+@pytest.mark.parametrize("independent", [False, True])
+def test_units(ctx, specs, dt, plain_units, units, units_independent, independent):  # noqa: F811
     from paper_2501_10653_gb300 import iqa
     code = {"f32": 0, "f16": 1, "bf16": 2}[dt]
+    flags = iqa.IQA_PLAN_INDEPENDENT if independent else iqa.IQA_PLAN_GRAPH
     b = Batch(specs, dtype=dt, seed=62)
-    small = _run(ctx, b, dtype_code=code)
+    small = _run(ctx, b, flags=flags, dtype_code=code)
     got = [b.results(i) for i in range(len(specs))]
     c = small.config
     shape = {"threads": c.threads, "unit_kpx": c.unit_kpx}
     assert sum(iqa.iqa_plan_unit_shape(code, N, NT, shape)[2] for N, NT in specs) == plain_units
-    assert small.total_units == units
-    plain = _plan_with_shape(ctx, b, shape, dtype_code=code)
+    assert small.total_units == (units_independent if independent else units)
+    plain = _plan_with_shape(ctx, b, shape, flags=flags, dtype_code=code)
     assert plain.total_units == plain_units
     for i in range(len(specs)):
         for u, v in zip(got[i], b.results(i)):
