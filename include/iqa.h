@@ -644,9 +644,10 @@ typedef enum {
      * call writes (a stream of calls over other outputs, or the same call
      * repeated, qualifies).  Each CTA then loads and reduces its pixels while
      * that kernel drains, and waits for it only before writing its maps, so
-     * the call's writes and completion still follow it.  Breaking the promise
-     * gives wrong maps, not a fault.  0 (default): every CTA waits before its
-     * first access. */
+     * the call's writes and completion still follow it.  Calls whose tiles are
+     * not whole 16-byte vectors, and calls split over the GPU (iqa_get_config),
+     * wait as with 0.  Breaking the promise gives wrong maps, not a fault.  0
+     * (default): every CTA waits before its first access. */
     IQA_OPT_INDEPENDENT_CALLS = 3
 } iqa_option;
 

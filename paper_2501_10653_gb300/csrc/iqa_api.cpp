@@ -138,11 +138,14 @@ bool any_config_valid(int N, int NT, iqa_dtype dtype, const TileConfig &c,
     return false;
 }
 
-// CTAs per SM that the one-wave rule below counts with.  A launch shape fixes
-// the order of a tile's sums, so these numbers are part of a map's bits: they
-// are those of the kernel whose shapes were swept for the rule (96 to 120
-// registers a thread with eight FP32 vectors in flight, 46 to 72 otherwise) and
-// stay as they are whatever the kernel's registers or shared memory become.
+// CTAs per SM that the rule below counts with.  A launch shape fixes the order
+// of a tile's sums, so these numbers are part of a map's bits: they are those of
+// the kernel whose shapes were swept for the rule (96 to 120 registers a thread
+// with eight FP32 vectors in flight, 46 to 72 otherwise) and stay as they are
+// whatever the kernel's registers or shared memory become.  For FP32 from
+// registers they still are what an SM holds.  For 16 bits in batches of eight
+// they no longer are: the ring kernel holds four or six CTAs of 128 threads (ten
+// here), two of 256 (four) and one or two of 512.
 static int shape_residency(iqa_dtype dtype, const TileConfig &c)
 {
     if (dtype == IQA_F32) {
@@ -216,11 +219,12 @@ TileConfig default_config(int N, int NT, iqa_dtype dtype, bool aligned,
     return c;
 }
 
-// One wave: when the units of a one-pair launch need more than one but at
-// most two waves of resident CTAs (the last wave then runs a fraction of the
-// GPU and its ramp and tail are paid twice), units twice as wide that fit one
-// wave are used instead (N=2048, N_T=64: 512 CTAs of two tiles, 12.96 against
-// 14.3 us per isolated launch).  A map comes out of the same launch shape, and
+// One wave, counted with shape_residency: when the units of a one-pair launch
+// need more than one but at most two waves of CTAs (the last wave then runs a
+// fraction of the GPU and its ramp and tail are paid twice), units twice as wide
+// that fit one wave are used instead (N=2048, N_T=64 FP32: 512 CTAs of two tiles,
+// 12.96 against 14.3 us per isolated launch).  For 16-bit batches of eight, where
+// the count is not what an SM holds, it is a rule on unit counts and no more.  A map comes out of the same launch shape, and
 // so bit for bit the same, in every call, whichever maps are requested.
 static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, TileConfig c)
 {
@@ -251,8 +255,8 @@ static TileConfig fit_one_wave(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, Til
             }
         }
     }
-    // A grid that fills at most half of the resident slots leaves load
-    // slots unused: wider CTAs put more loads in flight at once, as long as
+    // A grid that fills at most half of the slots counted leaves load slots
+    // unused: wider CTAs put more loads in flight at once, as long as
     // every thread keeps a full batch of 8 vectors and the grid still fits
     // one wave (N=2048, N_T=128: 256 CTAs of 256 threads, 8.3 against 10.2 us
     // per isolated launch).

@@ -538,8 +538,9 @@ __device__ __forceinline__ void accumulate_unit(const T *__restrict__ xu,
 // the same elements in the same batches, with the offset stepped instead of
 // formed from row and column, and no test per element but in the last batch.
 // The loads are volatile so that a batch's are issued before its arithmetic.
-// This path is bound by instruction issue: with a 64-bit offset multiplied out
-// and a bound tested for every element it took 56 instructions per 32 elements.
+// This path is bound by instruction issue and the latency of its short loads:
+// with a 64-bit offset multiplied out and a bound tested for every element it
+// took 56 instructions per 32 elements, now 33 (N = 3000, N_T = 75 FP32).
 // Back to back, before and after: N = 3000, N_T = 75 FP32 19.4 and 15.3 us, FP16
 // 19.7 and 13.4; N = 2001, N_T = 69 BF16 22.7 and 8.8; N = 8001, N_T = 63 BF16
 // 218 and 92.  (Copies to shared memory, of aligned vectors by the whole CTA or

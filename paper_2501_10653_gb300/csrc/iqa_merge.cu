@@ -9,9 +9,10 @@
 // sum the four per-tile sums of each block in FP64, in an order fixed by the
 // launch shape (so results repeat bit for bit), and apply Eq. 1 / Eq. 2 once.
 //
-// What bounds the kernels is the FP64 pipe (busy half to three quarters of the
-// time), then the 32 bytes read per tile: an FP64 instruction holds an SM's
-// pipe for about 16 cycles, whatever the number of its active lanes.  So sums
+// What bounds the kernels is the FP64 pipe (T = 512, m = 8: busy half of the
+// cycles in which an SM works), then the 32 bytes read per tile: an FP64
+// instruction holds an SM's pipe for about 16 cycles, whatever the number of its
+// active lanes.  So sums
 // are formed with full warps, and the two quotients of a merged tile in float32
 // with one FP64 residual each, to the same rounding (ratio()).  By block width m, measured back to
 // back with all outputs, in us, against one thread (m <= 4), warp (m <= 90) or

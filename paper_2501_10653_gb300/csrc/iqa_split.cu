@@ -13,8 +13,8 @@ namespace iqa {
 
 // blockIdx.y = unit, blockIdx.x = sum * (TH / kSplitThreads) + slice: a GPU
 // thread per thread of the unit adds its batches of one sum in order, and the
-// warp's totals go through the tree of reduce_unit.  Bound by the chain, about
-// 16 cycles a batch (N = N_T = 4096 FP32: 128 batches, 1 us), as long as its
+// warp's totals go through the tree of reduce_unit.  Bound by the chain, four
+// dependent additions a batch (N = N_T = 4096 FP32: 128 batches), as long as its
 // loads arrive in time: AHEAD of them are on their way while the previous AHEAD
 // are added.  Eight at a time, waited for each time, left the whole N = N_T =
 // 4096 call at 51.5 us (32.7 with 32 ahead); units of few batches take 8, whose
@@ -241,8 +241,8 @@ void credit_memory(iqa_ctx *ctx, size_t bytes)
 // Whether the units of shape c (one-pair kernel) leave so many SMs idle for so
 // long that three launches are faster.  Measured one-pair kernel against split,
 // in us, back to back / a call alone:
-//   * element order (256 threads, 4 or 2 bytes a load), which runs one CTA an SM
-//     up to 152 units (run_pair): the split takes its three launches and the
+//   * element order (256 threads, 4 or 2 bytes a load), spread one to an SM
+//     up to 152 units (spread_smem): the split takes its three launches and the
 //     image's bytes, the units the time of one.  N = 401, one tile of 161K pixels:
 //     31.3 / 45 against 8.6 / 23; tiles of N_T = 211 (45K): 9 units 13.1 / 24
 //     against 9.9 / 25, 36 18.3 / 24 and 15.0 / 28, 64 15.1 / 29 and 17.9 / 30, 144

@@ -17,9 +17,9 @@
 //      the units of a tile in rank order, Eq. 1 and Eq. 2.
 // The three launches overlap by programmatic dependent launch.  Bound by the
 // first one's reads and, for small images, by the launches (about 8 us in all).
-// Against the one-pair kernel's CTAs: N = N_T = 4096 FP32 31.4 us against 246,
-// FP16 20.2 against 333 (140 with the ring); N = N_T = 8192 FP32 104 against
-// 963; N = 4095, N_T = 1365 FP32 (elements) 45 against 167.
+// Against the one-pair kernel's CTAs: N = N_T = 4096 FP32 31.4 us against 193,
+// FP16 20.5 against 137; N = N_T = 8192 FP32 104 against 734; N = 4095, N_T = 1365
+// FP32 (elements) 45 against 100.
 #pragma once
 
 #include "iqa_internal.h"
