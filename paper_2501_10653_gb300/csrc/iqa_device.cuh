@@ -133,11 +133,25 @@ template <> struct Elem<__half> { static constexpr int VEC = 8; };
 template <> struct Elem<__nv_bfloat16> { static constexpr int VEC = 8; };
 
 // 16-byte asynchronous copy to shared memory, past L1, with the same L2
-// prefetch hint.
-__device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
+// prefetch hint.  EVICT: the line is the first that L2 gives up.  Pixels are read
+// once, and read without it they push out of L2 what the kernel that made the
+// images left there, before the call gets to it.  First pass on images just
+// made, in us, without and with: N = 8192, N_T = 64 FP32 110 and 100 (from
+// registers, whose loads allocate nothing in L1, 103), N = 6144 74.5 and 67.1;
+// BF16 N = 5760 48.6 and 46.6; back to back the same (75.7 and 75.8).
+template <bool EVICT> __device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
 {
-    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src)
-                 : "memory");
+    if constexpr (EVICT) {
+        unsigned long long policy;
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+        asm volatile("cp.async.cg.shared.global.L2::cache_hint.L2::256B [%0], [%1], 16, %2;" ::"r"(
+                         dst),
+                     "l"(src), "l"(policy)
+                     : "memory");
+    } else {
+        asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src)
+                     : "memory");
+    }
 }
 
 // Starts a copy of the whole 16-byte pieces inside [p, p + bytes) to L2.  A hint:
@@ -377,7 +391,8 @@ struct Kahan {
 // 61 us, 51 with the ring), and every batch drains the pipeline at its end.
 //   ring    shared address of this thread's first slot; a ring entry is
 //           THREADS slots of x, then THREADS slots of y
-template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B,
+//   EVICT   the copies' hint to L2 (copy_async16)
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B, bool EVICT,
           typename Sink>
 __device__ __forceinline__ void sum_vectors_ring(const T *__restrict__ xu,
                                                  const T *__restrict__ yu, long long N, int LPU,
@@ -393,8 +408,8 @@ __device__ __forceinline__ void sum_vectors_ring(const T *__restrict__ xu,
     const long long wrap = N - (long long)LPU * VEC;  // extra step past a row's end
     long long off = (long long)row * N + (long long)col * VEC;
     const auto issue = [&](uint32_t slot) {
-        copy_async16(slot, xu + off);
-        copy_async16(slot + IMAGE, yu + off);
+        copy_async16<EVICT>(slot, xu + off);
+        copy_async16<EVICT>(slot + IMAGE, yu + off);
         off += step;
         col += dcol;
         if (col >= LPU) {
@@ -461,7 +476,7 @@ __host__ __device__ __forceinline__ int items_from(int first, int stride, int to
 // Streams one unit (RH rows x LPU vectors) through the ring and returns this
 // thread's four sums: vectors tid, tid + THREADS, ..., each batch added with
 // compensation to the thread's totals.
-template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B>
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B, bool EVICT>
 __device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
                                                      const T *__restrict__ yu, long long N,
                                                      int RH, int LPU, float C1f, uint32_t ring,
@@ -469,7 +484,7 @@ __device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
 {
     const int tid = threadIdx.x;
     Kahan ka, kb, kx, ky;
-    sum_vectors_ring<T, VEC, ILP, THREADS, DEPTH, DO_A, DO_B>(
+    sum_vectors_ring<T, VEC, ILP, THREADS, DEPTH, DO_A, DO_B, EVICT>(
         xu, yu, N, LPU, tid, THREADS, items_from(tid, THREADS, RH * LPU), C1f, ring,
         [&](float a, float b, float x, float y) {
             if (DO_A) ka.add(a);

@@ -12,11 +12,11 @@
 // What bounds the kernels is the FP64 pipe (T = 512, m = 8: busy half of the
 // cycles in which an SM works), then the 32 bytes read per tile: an FP64
 // instruction holds an SM's pipe for about 16 cycles, whatever the number of its
-// active lanes.  So sums
-// are formed with full warps, and the two quotients of a merged tile in float32
-// with one FP64 residual each, to the same rounding (ratio()).  By block width m, measured back to
-// back with all outputs, in us, against one thread (m <= 4), warp (m <= 90) or
-// cluster per merged tile with 64-bit index divisions and FP64 quotients:
+// active lanes.  So sums are formed with full warps, and the two quotients of a
+// merged tile in float32 with one FP64 residual each, to the same rounding
+// (ratio()).  By block width m, measured back to back with all outputs, in us,
+// against one thread (m <= 4), warp (m <= 90) or cluster per merged tile with
+// 64-bit index divisions and FP64 quotients:
 //   * m <= 4: a thread per merged tile, its tiles in 32-byte loads (T = 512: m =
 //     1 9.4 against 17.7, m = 2 11.7 / 23.2, m = 4 6.9 / 11.3; without a stated
 //     residency the compiler kept 32 registers and loads waited: m = 2 15.6);
