@@ -364,12 +364,25 @@ static int prefetch_ctas(iqa_ctx *ctx, const TileArgs &a, const TileConfig &c, i
 }
 
 // The units of a one-pair launch that fall to an SM, 0 for less than a quarter.
+// For the element units of clusters, which are spread by it (kSpreadMost), the
+// CTAs an SM has to hold for all clusters to find a place at once: a cluster stays
+// inside a GPC, here of 20 SMs and a last one of 12, so that 49 clusters of three
+// or 16 of seven do not fit one CTA an SM (N = 1134, N_T = 162 FP32: 11.9 us spread to
+// one an SM and 8.4 free; N = 2324, N_T = 581 37.7 and 24.8).
 static int units_per_sm(iqa_ctx *ctx, int N, int NT, const TileConfig &c)
 {
+    constexpr long long kGpc = 20;
     const long long T = N / NT, units = T / c.TX * T * c.S;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
     if (4 * units <= sms) return 0;
-    return (int)std::min<long long>((units + sms - 1) / sms, 1 << 30);
+    long long k = (units + sms - 1) / sms;
+    if (c.vec == 1 && c.S > 1) {
+        const auto clusters = [&](long long ctas) {
+            return sms / kGpc * (kGpc * ctas / c.S) + sms % kGpc * ctas / c.S;
+        };
+        while (k < 8 && clusters(k) < units / c.S) ++k;
+    }
+    return (int)std::min<long long>(k, 1 << 30);
 }
 
 // One pair, arguments checked: the pinned launch shape if there is one, else

@@ -1,7 +1,8 @@
 """Element-order launches of few units (needs a GPU), which ask for shared memory
 so that no SM holds more than their even share: unit counts around a quarter of
-152 SMs and around one, two and three units per SM, alone and back to back on
-outputs that differ, against the oracle.  Tolerance: tests/parity.py."""
+152 SMs and around one, two and three units per SM, and clusters that fit one CTA
+an SM or do not, alone and back to back on outputs that differ, against the
+oracle.  Tolerance: tests/parity.py."""
 import numpy as np
 import pytest
 
@@ -22,13 +23,15 @@ def ctx():
     iqa.iqa_destroy(h)
 
 
-# T^2 = 36, 49, 144, 169, 289, 324, 441, 484 units
+# T^2 = 36, 49, 144, 169, 289, 324, 441, 484 units of one CTA; clusters of two, three
+# and seven: 98 and 162, 147 and 300, 63 and 112 CTAs
 @pytest.mark.parametrize("dt", ["f32", "f16", "bf16"])
-@pytest.mark.parametrize("T", [6, 7, 12, 13, 17, 18, 21, 22])
-def test_few_element_units(ctx, orc, dt, T):
+@pytest.mark.parametrize("T,NT", [(6, 33), (7, 33), (12, 33), (13, 33), (17, 33), (18, 33),
+                                  (21, 33), (22, 33), (7, 202), (9, 202), (7, 177), (10, 177),
+                                  (3, 301), (4, 301)])
+def test_few_element_units(ctx, orc, dt, T, NT):
     import torch
     from paper_2501_10653_gb300 import iqa
-    NT = 33
     N = NT * T
     x, y = synth.paper_pair(N=N, dtype=dt)
     dx, dy = parity.to_device(x), parity.to_device(y)
