@@ -246,12 +246,17 @@ void credit_memory(iqa_ctx *ctx, size_t bytes)
 //     image's bytes, the units the time of one.  N = 401, one tile of 161K pixels:
 //     31.3 / 45 against 8.6 / 23; tiles of N_T = 211 (45K): 9 units 13.1 / 24
 //     against 9.9 / 25, 36 18.3 / 24 and 15.0 / 28, 64 15.1 / 29 and 17.9 / 30, 144
-//     20.0 / 30 and 23.3 / 39.  So fewer units the smaller they are: 4.8M pixels
-//     and a pixel for each unit below 152.
+//     20.0 / 30 and 23.3 / 39.  So fewer units the smaller they are: 192 less one
+//     for each unit, times a unit's pixels, above 4.2M for 16 bits, 3.4M for FP32,
+//     which leaves to the split what it is faster at with inputs in L2 (N_T = 233,
+//     100 of 54K FP32 23.1 / 33 and 20.2 / 34; N_T = 609, 112 of 53K FP16 24.6 / 34
+//     and 22.4 / 37) or not (N_T = 422, 128 of 89K FP32 37.9 / 51 and 33.9 / 48; N_T =
+//     801, 147 of 214K 100 / 106 and 74.7 / 89; N_T = 298, 128 of 44K 21.4 / 33 and
+//     21.5 / 36).
 //   * vectors: not from one unit per SM on (FP32 N = 3072, N_T = 512, 288 units:
 //     18.5 / 26 against 20.5 / 31; N = 6200, N_T = 1240: 55.7 / 69 and 62.2 / 77; FP16
 //     N = 8192, N_T = 1024, 512 units: 42.8 / 57 and 57.3 / 68).  With a third to two
-//     thirds of a unit per SM the clusters find an SM for each CTA, and the
+//     thirds of a unit per SM full clusters find an SM for each CTA, and the
 //     split pays for few shapes (72 units of 131K pixels: FP32 18.7 / 30 against
 //     20.7 / 31, FP16 12.8 / 25 and 15.4 / 28; of 524K FP16 38.3 / 52 and 37.0 / 48);
 //     with two thirds to one it pays again (128 units of 131K: FP32 35.0 / 42
@@ -271,9 +276,12 @@ bool split_pays(iqa_ctx *ctx, int N, int NT, iqa_dtype dtype, const TileConfig &
     const long long T = N / NT, units = T * T * c.S;
     const long long unit_px = (long long)NT * NT / c.S;
     const long long sms = ctx->num_sms > 0 ? ctx->num_sms : 152;
+    if (c.vec == 1) {
+        const long long least = dtype == IQA_F32 ? 3400000 : 4200000;
+        return unit_px >= 40000 && (sms + sms / 4 + 2 - units) * unit_px > least;
+    }
     if (units >= sms || unit_px < 32768) return false;
-    if (c.vec == 1) return unit_px >= 40000 && (sms - units) * unit_px > 4800000;
-    const bool one_an_sm = 3 * units > sms && 3 * units <= 2 * sms;
+    const bool one_an_sm = c.S == kMaxCluster && 3 * units > sms && 3 * units <= 2 * sms;
     if (dtype != IQA_F32) return unit_px >= (one_an_sm ? 400000 : 100000);
     if (unit_px >= 100000) return !one_an_sm;
     return N % 512 == 0 || (units <= 16 && unit_px >= 50000);

@@ -24,9 +24,11 @@ def contexts():
 
 # (dtype, N, N_T, elements that y lies off a 16-byte boundary, split).  Vectors:
 # units of 100K pixels (16 bits); 32K where rows lie 2 KB apart, 50K where units
-# are at most 16, else 100K (FP32); none of either with a third to two thirds of
-# a unit per SM, but of 16 bits from 400K pixels on, nor with one and more.
-# Elements: 40K pixels, and 4.8M pixels and more for all units below 152.
+# are at most 16, else 100K (FP32); none of either in clusters of eight with a
+# third to two thirds of a unit per SM, but of 16 bits from 400K pixels on, nor
+# with one and more.
+# Elements: 40K pixels, and 192 less the units, times a unit's pixels, above 4.2M
+# (16 bits) or 3.4M (FP32).
 CASES = [
     ("f32", 1536, 1536, 0, True), ("f32", 2048, 1024, 0, True), ("f32", 800, 800, 0, True),
     ("f32", 600, 600, 0, False), ("f32", 2480, 1240, 0, True), ("f32", 1600, 800, 0, False),
@@ -34,10 +36,12 @@ CASES = [
     ("f32", 2560, 512, 0, False), ("f32", 2500, 500, 0, False), ("f32", 1024, 256, 0, False),
     ("f32", 1536, 1536, 1, True), ("f32", 1031, 1031, 0, True), ("f32", 2022, 1011, 0, True),
     ("f32", 1626, 542, 0, True), ("f32", 1533, 511, 0, False), ("f32", 844, 211, 0, True),
-    ("f32", 1477, 211, 0, False),
+    ("f32", 1477, 211, 0, True), ("f32", 2321, 211, 0, False), ("f32", 1788, 298, 0, True),
+    ("f32", 2384, 298, 0, False), ("f32", 2052, 684, 0, False), ("f32", 3852, 1284, 0, True),
     ("f16", 1536, 1536, 0, True), ("f16", 1600, 800, 0, False), ("f16", 1536, 512, 0, False),
     ("f16", 3072, 1024, 0, False), ("f16", 1031, 1031, 0, True), ("f16", 1600, 800, 3, True),
-    ("f16", 1533, 511, 0, False),
+    ("f16", 1533, 511, 0, False), ("f16", 1477, 211, 0, True), ("f16", 2384, 298, 0, False),
+    ("f16", 1652, 826, 0, True),
     ("bf16", 2048, 1024, 0, True), ("bf16", 1626, 542, 0, True), ("bf16", 1536, 512, 0, False),
 ]
 
