@@ -133,25 +133,35 @@ template <> struct Elem<__half> { static constexpr int VEC = 8; };
 template <> struct Elem<__nv_bfloat16> { static constexpr int VEC = 8; };
 
 // 16-byte asynchronous copy to shared memory, past L1, with the same L2
-// prefetch hint.  EVICT: the line is the first that L2 gives up.  Pixels are read
-// once, and read without it they push out of L2 what the kernel that made the
-// images left there, before the call gets to it.  First pass on images just
-// made, in us, without and with: N = 8192, N_T = 64 FP32 110 and 100 (from
-// registers, whose loads allocate nothing in L1, 103), N = 6144 74.5 and 67.1;
-// BF16 N = 5760 48.6 and 46.6; back to back the same (75.7 and 75.8).
-template <bool EVICT> __device__ __forceinline__ void copy_async16(uint32_t dst, const void *src)
+// prefetch hint; HINT: with a policy for L2 (l2_policy).
+template <bool HINT>
+__device__ __forceinline__ void copy_async16(uint32_t dst, const void *src,
+                                             unsigned long long policy)
 {
-    if constexpr (EVICT) {
-        unsigned long long policy;
-        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    if constexpr (HINT)
         asm volatile("cp.async.cg.shared.global.L2::cache_hint.L2::256B [%0], [%1], 16, %2;" ::"r"(
                          dst),
                      "l"(src), "l"(policy)
                      : "memory");
-    } else {
+    else
         asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src)
                      : "memory");
-    }
+}
+
+// Policy of the copies of a pair of N x N images: lines of large pairs are the
+// first that L2 (129 MB) gives up.  Pixels are read once, and such a pair would
+// push out of L2 what the kernel that made the images left there, before the call
+// gets to it.  First pass on images just made, in us, without and with: N = 8192,
+// N_T = 64 FP32 110 and 100 (from registers, whose loads allocate nothing in L1,
+// 103), N = 6144 74.5 and 67.1; BF16 N = 5760 48.6 and 46.6; back to back the same
+// (75.7 and 75.8).  Pairs that L2 holds may be read from it again (N = 3200, N_T =
+// 32 FP32, three pairs in turn, 14.1 and 14.7).
+template <typename T> __device__ __forceinline__ unsigned long long l2_policy(long long N)
+{
+    unsigned long long first, normal;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
+    return 2 * N * N * (long long)sizeof(T) >= 120LL << 20 ? first : normal;
 }
 
 // Starts a copy of the whole 16-byte pieces inside [p, p + bytes) to L2.  A hint:
@@ -391,8 +401,8 @@ struct Kahan {
 // 61 us, 51 with the ring), and every batch drains the pipeline at its end.
 //   ring    shared address of this thread's first slot; a ring entry is
 //           THREADS slots of x, then THREADS slots of y
-//   EVICT   the copies' hint to L2 (copy_async16)
-template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B, bool EVICT,
+//   HINT    the copies carry l2_policy
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B, bool HINT,
           typename Sink>
 __device__ __forceinline__ void sum_vectors_ring(const T *__restrict__ xu,
                                                  const T *__restrict__ yu, long long N, int LPU,
@@ -407,9 +417,10 @@ __device__ __forceinline__ void sum_vectors_ring(const T *__restrict__ xu,
     const long long step = (long long)drow * N + (long long)dcol * VEC;
     const long long wrap = N - (long long)LPU * VEC;  // extra step past a row's end
     long long off = (long long)row * N + (long long)col * VEC;
+    const unsigned long long policy = HINT ? l2_policy<T>(N) : 0;
     const auto issue = [&](uint32_t slot) {
-        copy_async16<EVICT>(slot, xu + off);
-        copy_async16<EVICT>(slot + IMAGE, yu + off);
+        copy_async16<HINT>(slot, xu + off, policy);
+        copy_async16<HINT>(slot + IMAGE, yu + off, policy);
         off += step;
         col += dcol;
         if (col >= LPU) {
@@ -476,7 +487,7 @@ __host__ __device__ __forceinline__ int items_from(int first, int stride, int to
 // Streams one unit (RH rows x LPU vectors) through the ring and returns this
 // thread's four sums: vectors tid, tid + THREADS, ..., each batch added with
 // compensation to the thread's totals.
-template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B, bool EVICT>
+template <typename T, int VEC, int ILP, int THREADS, int DEPTH, bool DO_A, bool DO_B, bool HINT>
 __device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
                                                      const T *__restrict__ yu, long long N,
                                                      int RH, int LPU, float C1f, uint32_t ring,
@@ -484,7 +495,7 @@ __device__ __forceinline__ void accumulate_unit_ring(const T *__restrict__ xu,
 {
     const int tid = threadIdx.x;
     Kahan ka, kb, kx, ky;
-    sum_vectors_ring<T, VEC, ILP, THREADS, DEPTH, DO_A, DO_B, EVICT>(
+    sum_vectors_ring<T, VEC, ILP, THREADS, DEPTH, DO_A, DO_B, HINT>(
         xu, yu, N, LPU, tid, THREADS, items_from(tid, THREADS, RH * LPU), C1f, ring,
         [&](float a, float b, float x, float y) {
             if (DO_A) ka.add(a);

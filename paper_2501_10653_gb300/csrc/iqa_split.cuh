@@ -17,7 +17,7 @@
 //      the units of a tile in rank order, Eq. 1 and Eq. 2.
 // The three launches overlap by programmatic dependent launch.  Bound by the
 // first one's reads and, for small images, by the launches (about 8 us in all).
-// Against the one-pair kernel's CTAs: N = N_T = 4096 FP32 30.4 us against 193,
+// Against the one-pair kernel's CTAs: N = N_T = 4096 FP32 30.0 us against 193,
 // FP16 20.5 against 137; N = N_T = 8192 FP32 104 against 734; N = 4095, N_T = 1365
 // FP32 (elements) 45 against 100.
 #pragma once
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kSplitThreads) iqa_split_sums_kernel(const Spl
         out += 4 * p.TH;
     };
     if constexpr (VEC > 1) {
-        // (the hint: N = N_T = 4096 FP32 31.4 us without and 30.4 with, FP16 20.3 and
+        // (the policy: N = N_T = 4096 FP32 31.4 us without and 30.0 with, FP16 20.3 and
         // 20.7)
         sum_vectors_ring<T, VEC, kSplitIlp, kSplitThreads, kSplitDepth, DO_A, DO_B, VEC == 4>(
             xu, yu, N, p.t.LPU, first, p.TH, n, p.t.C1f,

@@ -89,11 +89,11 @@ template <int VEC> inline bool use_ring(const TileArgs &p, int ilp, int rows)
 // against 43.3), four 1-2% slower.
 __host__ __device__ constexpr int ring_depth(int threads) { return threads == 512 ? 4 : 8; }
 
-// Whether the ring's copies are the first that L2 gives up (copy_async16): FP32,
-// and 16 bits with six CTAs.  The 16-bit build for four then takes 118 registers in
+// Whether the ring's copies carry a policy for L2 (l2_policy): FP32, and 16 bits
+// with six CTAs.  The 16-bit build for four then takes 118 registers in
 // place of 102 and is 1-2% slower back to back (N = 8192, N_T = 128 FP16 43.8 and
 // 44.3), though faster on images just made (71.6 and 68.6).
-template <int VEC, int CTAS> constexpr bool kEvictFirst = VEC == 4 || CTAS == 6;
+template <int VEC, int CTAS> constexpr bool kL2Hint = VEC == 4 || CTAS == 6;
 
 // Resident CTAs to compile for.  Left to itself the compiler aims at a residency
 // of its own and sinks loads between their arithmetic for it; stated, it keeps a
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(THREADS, CTAS)
     {
         if constexpr (VEC > 1 && STREAMED)
             accumulate_unit_ring<T, VEC, ILP, THREADS, ring_depth(THREADS), DO_A, DO_B,
-                                 kEvictFirst<VEC, CTAS>>(
+                                 kL2Hint<VEC, CTAS>>(
                 xu, yu, p.N, p.RH, p.LPU, p.C1f,
                 (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * 16, acc);
         else if constexpr (STREAMED)
